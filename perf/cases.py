@@ -246,8 +246,8 @@ def _haar(kin, kout, n, gen, dtype):
     """Variant outputs [4^k, 2^(n + kout)] of a random isometry from the incoming wires to the data and outgoing ones."""
     ct = torch.complex128 if dtype == torch.float64 else torch.complex64
     amp = torch.randn(1 << kin, 1 << (n + kout), dtype=ct, device="cuda", generator=gen)
-    low = torch.linalg.cholesky((amp @ amp.mH).to(torch.complex128))
-    amp = torch.linalg.inv(low).to(ct) @ amp
+    low = np.linalg.cholesky((amp @ amp.mH).to(torch.complex128).cpu().numpy())        # orthonormal rows
+    amp = torch.from_numpy(np.linalg.inv(low)).to("cuda", ct) @ amp
     init = torch.ones(1, 1, dtype=torch.complex128, device="cuda")
     for _ in range(kin):
         init = torch.kron(init, torch.tensor(_INIT, dtype=torch.complex128, device="cuda"))
