@@ -99,9 +99,10 @@ typedef struct {
    * added into the output (in FP64 for FP64 outputs).  0 = no slicing. */
   int32_t slice_edges;
   /* Selection (sqc_top_bins): 1 = hold one 32-bit key word per value in
-   * shared memory, one slice per SM, when they fit (up to ~7 million FP32
-   * or FP64 values on 152 SMs; one read of the input); 0 = always the
-   * streaming kernel. */
+   * shared memory, one slice per SM, up to 5 * 2^20 values (one read of the
+   * input); 0 = always the filtering kernel that larger inputs take (one
+   * read too: a sample bounds the k-th value, only values above the bound
+   * are kept). */
   int32_t select_resident;
   /* Merge pyramid (1 = on, default 0): after every attribution, also keep
    * the partial marginals of each A_i over its 1, 2, ..., n_i lowest

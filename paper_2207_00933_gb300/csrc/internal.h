@@ -279,6 +279,14 @@ size_t select_resident_smem(uint64_t n, int is_f64, int grid, uint64_t* per);
 cudaError_t launch_select_resident(void* work, int grid, const void* x, int is_f64, uint64_t n, int k,
                                    double threshold, unsigned long long* bins_out, double* probs_out, int* n_found,
                                    int* err, cudaStream_t s);
+// The same selection for inputs of any size, read once: a sample bounds the
+// k-th value from below and only the values above the bound are kept.  Same
+// workspace, grid = select_resident_grid() (> 0).  Up to kStreamMost values
+// (the FP32 ranking packs a 32-bit bin with the key).
+constexpr uint64_t kStreamMost = uint64_t(1) << 32;
+cudaError_t launch_select_stream(void* work, int grid, const void* x, int is_f64, uint64_t n, int k,
+                                 double threshold, unsigned long long* bins_out, double* probs_out, int* n_found,
+                                 int* err, cudaStream_t s);
 // one-time per-device kernel attributes (large shared memory for the sort)
 cudaError_t select_configure();
 constexpr int kSelectMaxK = 4096;

@@ -23,6 +23,7 @@
 #include <cstring>
 #include <limits>
 #include <mutex>
+#include <type_traits>
 
 #include "device_ops.cuh"
 
@@ -602,13 +603,13 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* ctl, unsigned n
 __device__ __forceinline__ int pass_hi(int p) { return 64 - kCBits * p; }
 __device__ __forceinline__ int pass_lo(int p) { const int l = 64 - kCBits * (p + 1); return l > 0 ? l : 0; }
 
-template <bool is_f64>
-__global__ void __launch_bounds__(kCoopThreads)
-select_coop_kernel(const void* x, int aligned, uint64_t n, unsigned long long key_thr, int k, int cap,
-                   CoopWork w, unsigned long long* bins_out, double* probs_out, int* n_found, int* err) {
-  pdl_wait();      // the previous kernel on the stream has completed
-  pdl_trigger();   // the next one may start launching
-  extern __shared__ unsigned shw[];               // [kCoopWarps][kCRadix]
+// The body, for a whole grid of THREADS-thread CTAs; shw: one histogram per
+// warp.  Also what the filtering kernel falls back to.
+template <bool is_f64, int THREADS>
+__device__ __forceinline__ void coop_select(const void* x, int aligned, uint64_t n, unsigned long long key_thr, int k,
+                                            int cap, const CoopWork& w, unsigned long long* bins_out,
+                                            double* probs_out, int* n_found, int* err, unsigned* shw) {
+  constexpr int kCoopWarps = THREADS / 32;
   __shared__ unsigned long long s_prefix, s_krem, s_take;
   __shared__ int s_bits, s_done;
   const unsigned nb = gridDim.x;
@@ -851,6 +852,16 @@ fail:
   if (threadIdx.x == 0 && err) atomicExch(err, 1);
 }
 
+template <bool is_f64>
+__global__ void __launch_bounds__(kCoopThreads)
+select_coop_kernel(const void* x, int aligned, uint64_t n, unsigned long long key_thr, int k, int cap,
+                   CoopWork w, unsigned long long* bins_out, double* probs_out, int* n_found, int* err) {
+  pdl_wait();      // the previous kernel on the stream has completed
+  pdl_trigger();   // the next one may start launching
+  extern __shared__ unsigned shw[];               // [kCoopWarps][kCRadix]
+  coop_select<is_f64, kCoopThreads>(x, aligned, n, key_thr, k, cap, w, bins_out, probs_out, n_found, err, shw);
+}
+
 
 // ---- shared-memory-resident cooperative selection --------------------------------
 // For inputs that fit in the shared memory of one CTA per SM (the usual
@@ -878,7 +889,9 @@ constexpr uint32_t kRBarrierLimit = 1u << 21;       // polls (~1-2 s) before a b
 
 struct ResWork {
   // [0] barrier word: arrivals (high 32 bits) and candidates (low 32 bits,
-  // added at the compaction barrier); [1] exits; [2] abort; [3] slots
+  // added at the compaction barrier); [1] exits; [2] abort; [3] slots;
+  // filtering kernel: [4] a CTA's candidate buffer ran over; [5] values
+  // equal to the filter's key
   unsigned long long* ctl;
   unsigned* hist;                 // [kRMaxPasses][kRRadix]
   unsigned long long* cand_key;   // [kMaxSort]
@@ -1447,22 +1460,313 @@ __device__ __forceinline__ void rank_candidates(const ResWork& w, unsigned nc, u
   }
 }
 
-// TAIL: the input is not read but computed -- the query's contraction
+// ---- filtering selection (inputs of any size) ------------------------------------
+// Larger inputs than the resident form holds are read ONCE: a sample of the
+// input gives a key tau that about a 500th of the values (and a few times k)
+// exceed, the CTAs stream the input keeping only those (key word and bin in
+// shared memory), and the refinement passes, compaction and ranking of the
+// resident kernel run on the kept values.  Exact whatever the sample says: if
+// fewer than k values exceed tau, the missing ones are ties of tau itself
+// (counted in the same pass, taken in ascending bin order) or the whole
+// selection falls back to the radix passes over the input (coop_select), as
+// it does when a CTA's buffer runs over.
+//
+// Every CTA reads the same sample (8192 values, once from HBM, then from L2)
+// and finds tau by itself, so the sample costs no grid barrier; and it ranks
+// only the largest value each of its threads read (16384 values ranked by
+// histograms took 12 us of 33 at 2^20).  Meanwhile the head of the input is
+// fetched.  The kept values need one histogram where digits of the key need
+// two or three: log-scaled buckets of the distance above tau.
+//
+// Bound: HBM, n x s B read once, plus ~20 us of sample, grid barriers (the
+// buckets and the compaction) and ranking.  2^26 FP32 values, k = 1024: 70 us
+// (the five reads of the radix passes: 650 us); FP64 118 us.
+constexpr unsigned kSampleChunks = 2;        // 4-value sample chunks per thread (inputs up to 2^27 values;
+constexpr unsigned kSampleChunksMost = 64;   // more for larger ones, so that the kept values fit)
+constexpr uint64_t kSampleSpan = 16;         // values per sampled chunk at least
+constexpr unsigned kSampleAbove = 16;        // sampled values above tau at least,
+constexpr unsigned kSampleAboveMost = 256;   // and at most (of kRThreads ranked)
+constexpr uint64_t kFilterAllBelow = uint64_t(1) << 18;   // inputs this small keep every value
+constexpr int kRing = 8;                     // vectors per thread on their way through shared memory
+constexpr int kHeadRounds = 12;              // rounds after the ring's fetched into L2 while the sample is read
+struct StreamArgs {
+  unsigned strata;            // sampled chunks (0: no sample, keep every value >= the threshold),
+  unsigned chunks;            // and how many of them a thread reads
+  uint64_t span;              // values per stratum
+  unsigned j;                 // tau = the j-th largest of the threads' largest sampled values
+  unsigned buf;               // kept values per CTA at most
+  CoopWork coop;              // workspace and
+  int coop_cap;               // bucket capacity of the fallback
+};
+struct NoSource {};
+
+// The sampled chunk of stratum s: a fixed pseudo-random multiple of 4 inside
+// it (a mixing function of the index, so that no period of the input lines
+// up with the sample).
+__device__ __forceinline__ uint64_t sample_at(unsigned s, uint64_t span) {
+  unsigned h = s * 0x9E3779B1u;
+  h ^= h >> 15;
+  h *= 0x85EBCA77u;
+  h ^= h >> 13;
+  const uint64_t room = span >> 2;           // chunks of 4 in a stratum
+  return uint64_t(s) * span + 4 * ((uint64_t(h) * room) >> 32);
+}
+
+// The sample's tau, found by every CTA alike from the same values: the
+// largest key that at least j threads' largest values reach, bit by bit (a
+// barrier that counts per bit; three 12-bit histograms took twice as long).
+// 0: at most j threads read a value >= the threshold, there is no tau.
+template <bool F64>
+__device__ __forceinline__ unsigned long long sample_tau(const void* x, int aligned, uint64_t n,
+                                                         unsigned long long key_thr64, const StreamArgs& S) {
+  using Key = typename std::conditional<F64, unsigned long long, unsigned>::type;
+  constexpr int KB = F64 ? 64 : 32;
+  const int tid = threadIdx.x;
+  Key key = 0;                                       // 0: excluded (no included value has it)
+  for (unsigned h0 = 0; h0 < S.chunks; h0 += 2) {
+    Chunk c[2];
+#pragma unroll
+    for (unsigned h = 0; h < 2; ++h) {
+      const unsigned s = (h0 + h) * unsigned(kRThreads) + unsigned(tid);
+      load_chunk<F64>(x, aligned, n, s < S.strata ? sample_at(s, S.span) & ~uint64_t(3) : n, key_thr64, &c[h]);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int q = 0; q < kVec; ++q) {
+        const Key k = c[h].ok[q] ? Key(c[h].key[q] >> (64 - KB)) : Key(0);
+        key = k > key ? k : key;
+      }
+  }
+  if (__syncthreads_count(key != 0) <= int(S.j)) return 0ull;
+  Key tau = 0;
+  for (int bit = KB - 1; bit >= 0; --bit) {
+    // FP64 values that FP32 holds too (the usual contents of FP64 bins) have
+    // an empty low word: one count instead of 32
+    if (F64 && bit == 31 && __syncthreads_count(key > tau) < int(S.j)) break;
+    const Key up = tau | (Key(1) << bit);
+    if (__syncthreads_count(key >= up) >= int(S.j)) tau = up;
+  }
+  return tau;
+}
+
+// The 16-byte vectors of the input that this thread tests: one per round,
+// rounds gridDim.x x kRThreads vectors apart, so that values that crowd
+// together in the input spread over the CTAs.
+__device__ __forceinline__ void ring_request(unsigned char* ring, const void* x, uint64_t vec, uint64_t vecs,
+                                             unsigned round) {
+  if (vec < vecs)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(uint32_t(__cvta_generic_to_shared(
+                     ring + (size_t(round % kRing) * kRThreads + threadIdx.x) * 16))),
+                 "l"(static_cast<const char*>(x) + vec * 16)
+                 : "memory");
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// The input's values whose key exceeds tau (and is not NaN), of the vectors
+// this CTA tests, appended to keys / cidx (key word, bin) in no particular
+// order; *s_cnt counts them (beyond buf: not kept), *s_eq the values equal
+// to tau.  Each thread reads its vectors through its own slots of a ring in
+// shared memory (cp.async, kRing - 1 ahead; no barrier): with 200 KB of
+// shared memory in use, plain loads are held to what little is left of L1
+// (4.8 TB/s against 6.9 at 2^26 values).  ring_request of the first kRing - 1
+// rounds precedes the call.
+template <bool F64>
+__device__ __forceinline__ void filter_input(const void* x, int aligned, uint64_t n, unsigned long long tau,
+                                             bool count_eq, unsigned buf, unsigned char* ring, unsigned* keys,
+                                             unsigned* cidx, unsigned* s_cnt, unsigned long long* s_eq) {
+  constexpr int V = F64 ? 2 : 4;
+  using Word = typename std::conditional<F64, unsigned long long, unsigned>::type;
+  const int tid = threadIdx.x, lane = tid & 31;
+  // keys in (tau, key of +infinity]: one subtraction and one comparison
+  const unsigned t32 = unsigned(tau), r32 = 0xff800000u - t32;
+  const unsigned long long r64 = 0xfff0000000000000ull - tau;
+  // tau's (high) word as a signed integer; below zero: test every value
+  const unsigned thi = F64 ? unsigned(tau >> 32) : t32;
+  const int tword = (thi & 0x80000000u) ? int(thi & 0x7fffffffu) : int(0x80000000u);
+  unsigned eq = 0;
+  auto test = [&](const Word (&bits)[V], uint64_t bin, int cnt) {
+    // the (high) words as signed integers are ordered as the values are from
+    // zero up: a maximum per vector, and the exact test only where it reaches
+    // tau's word (testing every value exactly took 20 instructions a value)
+    int top = int(unsigned(bits[0] >> (F64 ? 32 : 0)));
+#pragma unroll
+    for (int q = 1; q < V; ++q) {
+      const int b = int(unsigned(bits[q] >> (F64 ? 32 : 0)));
+      top = b > top ? b : top;
+    }
+    if (top < tword) return;
+    unsigned hits = 0;
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+      if (q >= cnt) break;
+      if constexpr (F64) {
+        const unsigned long long d = key_f64(__longlong_as_double((long long)bits[q])) - tau;
+        hits |= (d - 1ull < r64) ? 1u << q : 0u;
+        eq += d == 0ull;
+      } else {
+        const unsigned d = unsigned(key_f32(__uint_as_float(unsigned(bits[q]))) >> 32) - t32;
+        hits |= (d - 1u < r32) ? 1u << q : 0u;
+        eq += d == 0u;
+      }
+    }
+    if (hits) {
+      unsigned pos = atomicAdd(s_cnt, unsigned(__popc(hits)));
+#pragma unroll
+      for (int q = 0; q < V; ++q)
+        if ((hits >> q) & 1u) {
+          if (pos < buf) {
+            keys[pos] = unsigned((F64 ? key_f64(__longlong_as_double((long long)bits[q]))
+                                      : key_f32(__uint_as_float(unsigned(bits[q])))) >> 32);
+            cidx[pos] = unsigned(bin + q);
+          }
+          ++pos;
+        }
+    }
+  };
+  const uint64_t vecs = n / V, step = uint64_t(gridDim.x) * kRThreads;
+  uint64_t v = uint64_t(blockIdx.x) * kRThreads + tid;
+  if (aligned) {
+    for (unsigned r = 0; v < vecs; v += step, ++r) {
+      ring_request(ring, x, v + (kRing - 1) * step, vecs, r + kRing - 1);
+      asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 1) : "memory");
+      const unsigned char* slot = ring + (size_t(r % kRing) * kRThreads + tid) * 16;
+      Word bits[V];
+      if constexpr (F64) {
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(slot);
+        bits[0] = q.x; bits[1] = q.y;
+      } else {
+        const uint4 q = *reinterpret_cast<const uint4*>(slot);
+        bits[0] = q.x; bits[1] = q.y; bits[2] = q.z; bits[3] = q.w;
+      }
+      test(bits, v * V, V);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  } else {
+    for (; v < vecs; v += step) {
+      Word bits[V];
+#pragma unroll
+      for (int q = 0; q < V; ++q) bits[q] = static_cast<const Word*>(x)[v * V + q];
+      test(bits, v * V, V);
+    }
+  }
+  // the values after the last whole vector
+  if (blockIdx.x == 0 && tid == 0 && vecs * V < n) {
+    Word bits[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) bits[q] = vecs * V + q < n ? static_cast<const Word*>(x)[vecs * V + q] : Word(0);
+    test(bits, vecs * V, int(n - vecs * V));
+  }
+  if (count_eq) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) eq += __shfl_down_sync(0xffffffffu, eq, off);
+    if (lane == 0 && eq) atomicAdd(s_eq, (unsigned long long)eq);
+  }
+}
+
+// Ties of key tkey in the CTA's slice (full 64-bit keys for FP64), in
+// ascending bin order after every larger value: per-CTA counts, a grid
+// barrier, then an ordered scan of the slices that hold the first st.krem
+// of them.  Rare, out of line.  Returns false when the barrier gave up.
+template <bool F64>
+__device__ __noinline__ bool stream_tie_scan(const void* x, uint64_t start, uint64_t len, ResWork& w,
+                                             const ResState& st, unsigned* wcnt, unsigned nb, unsigned& bar) {
+  constexpr int E = 8;                               // consecutive values per thread and round
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned long long tkey = st.prefix;
+  auto tie = [&](uint64_t i) -> bool {
+    if constexpr (F64) return key_f64(static_cast<const double*>(x)[start + i]) == tkey;
+    else return (key_f32(static_cast<const float*>(x)[start + i]) >> 32) == tkey;
+  };
+  unsigned my = 0;
+#pragma unroll 8
+  for (uint64_t i = tid; i < len; i += kRThreads) my += tie(i);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) my += __shfl_down_sync(0xffffffffu, my, off);
+  if (lane == 0) wcnt[warp] = my;
+  __syncthreads();
+  if (tid == 0) {
+    unsigned c = 0;
+    for (int ww = 0; ww < kRWarps; ++ww) c += wcnt[ww];
+    w.tie_count[blockIdx.x] = c;
+  }
+  if (res_barrier(w.ctl, 1ull << 32, nb * ++bar) == 0ull) return false;
+  __shared__ unsigned long long tbase;
+  if (tid == 0) {
+    unsigned long long b = 0;
+    for (unsigned r = 0; r < blockIdx.x; ++r) b += __ldcg(w.tie_count + r);
+    tbase = b;
+  }
+  __syncthreads();
+  const unsigned long long need = st.krem, first = st.take - st.krem;
+  unsigned long long run = tbase;
+  for (uint64_t t0 = 0; t0 < len && run < need; t0 += uint64_t(kRThreads) * E) {
+    unsigned m = 0;
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+      const uint64_t i = t0 + uint64_t(tid) * E + q;
+      if (i < len && tie(i)) m |= 1u << q;
+    }
+    const unsigned mine = unsigned(__popc(m));
+    unsigned incl = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const unsigned o = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += o;
+    }
+    if (lane == 31) wcnt[warp] = incl;
+    __syncthreads();
+    unsigned before = 0, all = 0;
+    for (int ww = 0; ww < kRWarps; ++ww) {
+      if (ww < warp) before += wcnt[ww];
+      all += wcnt[ww];
+    }
+    unsigned long long rank = run + before + incl - mine;
+#pragma unroll
+    for (int q = 0; q < E; ++q)
+      if ((m >> q) & 1u) {
+        if (rank < need) {
+          w.cand_key[first + rank] = tkey;
+          w.cand_idx[first + rank] = start + t0 + uint64_t(tid) * E + q;
+        }
+        ++rank;
+      }
+    run += all;
+    __syncthreads();
+  }
+  return true;
+}
+
+// The radix passes over the whole input, for a filter that kept too few or
+// too many values.  Out of line: not on the common path.
+template <bool F64>
+__device__ __noinline__ void stream_fallback(const void* x, int aligned, uint64_t n, unsigned long long key_thr64,
+                                             int k, const StreamArgs& S, unsigned long long* bins_out,
+                                             double* probs_out, int* n_found, int* err, unsigned* shw) {
+  coop_select<F64, kRThreads>(x, aligned, n, key_thr64, k, S.coop_cap, S.coop, bins_out, probs_out, n_found, err, shw);
+}
+
+// SRC says where the values come from.
+// NoSource: the input, read whole into shared memory.
+// StreamArgs: the input, filtered (above).
+// TailArgs: the input is not read but computed -- the query's contraction
 // steps before the last run first (tail_pre_steps), then every CTA
 // computes its slice of the last step's bins itself (each bin one inner
 // product over the shared index, the operands in registers or shared
 // memory, the FP32 multiply-adds in the order of the per-step kernel, so
 // the bins are the same bit for bit), writes them to T.P in bin order and
 // keeps their keys -- the bins are written once and never read back.
-template <bool F64, bool TAIL>
+template <bool F64, class SRC>
 __global__ void __launch_bounds__(kRThreads, 1)
 select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, unsigned long long key_thr64, int k,
                        int cap, ResWork w, unsigned long long* bins_out, double* probs_out, int* n_found, int* err,
-                       TailArgs Tp) {
+                       SRC Tp) {
+  constexpr bool TAIL = std::is_same<SRC, TailArgs>::value;
+  constexpr bool STREAM = std::is_same<SRC, StreamArgs>::value;
   static_assert(!(F64 && TAIL), "the fused launch computes FP32 bins");
   // the fused launch reads its arguments from shared memory (one parallel
   // copy of the parameter block instead of scattered parameter loads)
-  const TailArgs* tq = &Tp;
+  const SRC* tq = &Tp;
   if constexpr (TAIL) {
     __shared__ __align__(16) TailArgs tsh;
     const unsigned long long* src = reinterpret_cast<const unsigned long long*>(&Tp);
@@ -1471,7 +1775,7 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
     __syncthreads();
     tq = &tsh;
   }
-  const TailArgs& T = *tq;
+  const SRC& T = *tq;
   // Shared memory holds one 32-bit word per value: the whole key of an FP32
   // value, the high word of the 64-bit key of an FP64 value (its low word
   // is read back from the input only for values whose high word equals the
@@ -1489,10 +1793,18 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned long long key_thr = F64 ? key_thr64 : (key_thr64 >> 32);
   const uint64_t start = uint64_t(blockIdx.x) * per;
-  const int cnt = int(start < n ? ((n - start) < per ? (n - start) : per) : 0);
-  // low word of the 64-bit key of value i of the slice (FP64 only)
+  const uint64_t len = start < n ? ((n - start) < per ? (n - start) : per) : 0;
+  int cnt = STREAM ? 0 : int(len);                  // values in keys
+  unsigned* cidx = keys;                            // STREAM: their bins
+  if constexpr (STREAM) cidx = keys + T.buf;
+  // bin of value i of keys
+  auto bin_of = [&](int i) -> uint64_t {
+    if constexpr (STREAM) return cidx[i];
+    else return start + uint64_t(i);
+  };
+  // low word of the 64-bit key of value i of keys (FP64 only)
   auto low_word = [&](int i) -> unsigned {
-    return unsigned(key_f64(static_cast<const double*>(x)[start + i]));
+    return unsigned(key_f64(static_cast<const double*>(x)[bin_of(i)]));
   };
   auto full_key = [&](int i, unsigned kk) -> unsigned long long {
     if constexpr (F64) return ((unsigned long long)kk << 32) | low_word(i);
@@ -1528,7 +1840,46 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
   // pass 0 with the load: keys of excluded values (NaN or below the
   // threshold) are stored as 0, which no included value has (the smallest
   // included key word is 0x007fffff for FP32, 0x000fffff for FP64)
-  if constexpr (TAIL) {
+  __shared__ unsigned s_kept;                       // STREAM: values the filter kept,
+  __shared__ unsigned long long s_eq, s_eq_all;     // values equal to tau seen by this CTA, by all
+  __shared__ unsigned s_over;                       // some CTA's buffer ran over
+  bool tau_thr = true, fallback = false;            // tau is the threshold; the filter's result cannot be used
+  unsigned long long tau = key_thr - 1;             // kept: keys above tau
+  if constexpr (STREAM) {
+    unsigned char* ring = reinterpret_cast<unsigned char*>(keys) + size_t(T.buf) * 8;
+    if (aligned) {
+      // the first rounds into the ring and the ones after them into L2, while
+      // the sample is read
+      const uint64_t vecs = n / (16 / (F64 ? 8 : 4)), step = uint64_t(nb) * kRThreads;
+      const uint64_t v0 = uint64_t(blockIdx.x) * kRThreads;
+      for (unsigned r = 0; r < unsigned(kRing - 1); ++r) ring_request(ring, x, v0 + tid + r * step, vecs, r);
+      if (tid < kHeadRounds && v0 + (tid + kRing) * step <= vecs)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const char*>(x) +
+                                                                      (v0 + (tid + kRing - 1) * step) * 16),
+                     "n"(kRThreads * 16)
+                     : "memory");
+    }
+    if (T.strata > 0) {
+      const unsigned long long t = sample_tau<F64>(x, aligned, n, key_thr64, T);
+      if (t != 0ull) {                               // (a sampled key: not below the threshold's)
+        tau = t;
+        tau_thr = false;
+      }
+    }
+    if (tid == 0) {
+      s_kept = 0u;
+      s_eq = 0ull;
+    }
+    for (int d = tid; d < kRRadix; d += kRThreads) sh[d] = 0u;
+    __syncthreads();
+    filter_input<F64>(x, aligned, n, tau, !tau_thr, T.buf, ring, keys, cidx, &s_kept, &s_eq);
+    __syncthreads();
+    cnt = int(s_kept < T.buf ? s_kept : T.buf);
+    if (tid == 0) {
+      if (s_kept > T.buf) atomicOr(w.ctl + 4, 1ull);
+      if (s_eq) atomicAdd(w.ctl + 5, s_eq);
+    }
+  } else if constexpr (TAIL) {
     __shared__ float2 tred[kRWarps];
     // the thread's bins summed as an unevaluated FP32 pair (hi + lo, each
     // addition error-free by Knuth's TwoSum), reduced over the CTA as pairs
@@ -1698,14 +2049,72 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
       }
     }
   }
+  // STREAM: what the CTAs' filters found, read after the first barrier;
+  // false: the filter's result cannot be used
+  [[maybe_unused]] auto filter_usable = [&]() -> bool {
+    if (tid == 0) {
+      s_over = unsigned(__ldcg(w.ctl + 4));
+      s_eq_all = __ldcg(w.ctl + 5);
+    }
+    __syncthreads();
+    return s_over == 0u;
+  };
+  // STREAM: bucket of a kept value's word above tau's, 0 the lowest
+  [[maybe_unused]] auto bucket_of = [&](unsigned kk) -> unsigned {
+    return unsigned(kRRadix - 1) - rank_bucket<false>(kk, F64 ? (tau >> 32) : tau);
+  };
+  bool by_bucket = false;                            // STREAM: decided by bucket (st.prefix)
+  if constexpr (STREAM) {
+    if (ok && !tau_thr) {
+      for (int i0 = 0; i0 < cnt; i0 += kRThreads) {
+        const int i = i0 + tid;
+        warp_hist_add(sh, i < cnt, i < cnt ? bucket_of(keys[i]) : 0u, lane);
+      }
+      __syncthreads();
+      unsigned* gh = w.hist + size_t(kRMaxPasses - 1) * kRRadix;
+      for (int d = tid; d < kRRadix; d += kRThreads) {
+        const unsigned v = sh[d];
+        if (v) atomicAdd(gh + d, v);
+      }
+      ok = res_barrier(w.ctl, 1ull << 32, nb * ++bar) != 0ull;
+      if (ok) fallback = !filter_usable();
+      if (ok && !fallback) {
+        res_decide(gh, 0, 0, false, k, cap, &st, wtot);
+        const unsigned long long above = st.take;    // min(k, kept values)
+        __syncthreads();
+        if (above < (unsigned long long)k) {
+          // fewer than k values above tau: the rest are ties of tau, or the
+          // sample misled
+          fallback = above + s_eq_all < (unsigned long long)k;
+          if (tid == 0 && !fallback) {
+            st.prefix = tau;
+            st.krem = (unsigned long long)k - above;
+            st.take = (unsigned long long)k;
+            st.lo = 0;
+            st.done = 3;
+          }
+        } else if (st.done == 1) {
+          by_bucket = true;
+        } else if (st.done == 0 && tid == 0) {       // the bucket does not fit: digits after all
+          st.prefix = 0ull;
+          st.krem = (unsigned long long)k;
+          st.lo = KB;
+        }
+        __syncthreads();
+      }
+    }
+  }
   // the refinement loop: flush, barrier, decide; then the next digit from
   // shared memory (and, for the low word of FP64 keys, from the input)
   for (int pass = 0; pass < kPasses; ++pass) {
+    if constexpr (STREAM) {
+      if (!ok || fallback || st.done) break;
+    }
     const int word = pass / 3;                      // 0: the (high) word in shared memory, 1: the low word
     const int hi_w = 32 - kRBits * (pass % 3);      // digit bits [lo_w, hi_w) of the word: 32-20, 20-8, 8-0
     const int lo_w = pass % 3 == 2 ? 0 : hi_w - kRBits;
     const int lo = ((F64 && word == 0) ? 32 : 0) + lo_w;   // bit position in the whole key
-    if (pass > 0) {
+    if (STREAM || pass > 0) {
       const unsigned long long pfx = st.prefix;
       const unsigned pfx_hi = F64 ? unsigned(pfx >> 32) : unsigned(pfx);
       const unsigned pfx_lo = unsigned(pfx);
@@ -1737,11 +2146,22 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
       if (v) atomicAdd(gh + d, v);
     }
     if (!(ok = res_barrier(w.ctl, 1ull << 32, nb * ++bar) != 0ull)) break;
+    if constexpr (STREAM) {
+      if (pass == 0 && tau_thr && (fallback = !filter_usable())) break;
+      if (pass == 0 && !tau_thr)                     // every CTA has read the buckets' histogram
+        for (uint64_t i = uint64_t(blockIdx.x) * kRThreads + tid; i < uint64_t(kRRadix); i += uint64_t(nb) * kRThreads)
+          w.hist[size_t(kRMaxPasses - 1) * kRRadix + i] = 0u;
+    }
     res_decide(gh, pass, lo, lo == 0, k, cap, &st, wtot);
     if (st.done) break;
   }
+  if constexpr (STREAM) {
+    if (ok && fallback)
+      stream_fallback<F64>(x, aligned, n, key_thr64, k, T, bins_out, probs_out, n_found, err,
+                           reinterpret_cast<unsigned*>(rsm));
+  }
   unsigned long long nc = 0;
-  if (ok) {
+  if (ok && !fallback) {
     const int done = st.done, lo = st.lo;
     const unsigned long long pfx = st.prefix;
     // compaction: values above the bucket, and the bucket itself unless it
@@ -1751,6 +2171,9 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
     auto takes = [&](int i, unsigned kk) -> bool {
       if (kk == 0) return false;
       if (done == 2) return true;
+      if constexpr (STREAM) {
+        if (by_bucket) return bucket_of(kk) >= unsigned(pfx);
+      }
       if (!F64 || lo >= 32) {
         // the bucket is decided within the word in shared memory
         const int l = F64 ? lo - 32 : lo;
@@ -1798,13 +2221,18 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
         const unsigned kk = keys[i];
         if (takes(i, kk)) {
           w.cand_key[r] = full_key(i, kk);
-          w.cand_idx[r] = start + i;
+          w.cand_idx[r] = bin_of(i);
           ++r;
         }
       }
     }
     __syncthreads();
-    if (done == 3) ok = tie_scan<F64>(w, keys, cnt, start, x, st, wcnt, nb, bar);
+    if (done == 3) {
+      if constexpr (STREAM)
+        ok = stream_tie_scan<F64>(x, start, len, w, st, wcnt, nb, bar);
+      else
+        ok = tie_scan<F64>(w, keys, cnt, start, x, st, wcnt, nb, bar);
+    }
     // the last barrier also sums the candidate counts into the low word
     if (ok) {
       const unsigned long long word = res_barrier(w.ctl, (1ull << 32) | cta_taken, nb * ++bar);
@@ -1834,11 +2262,11 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
     const unsigned long long take = st.take;
     if (st.done == 3) nc += st.krem;
     if (nc > (unsigned long long)kMaxSort) nc = kMaxSort;
-    const unsigned long long tmin = st.done == 2 ? key_thr : st.prefix;
-    if (nc > 0)
+    const unsigned long long tmin = st.done == 2 || by_bucket ? tau + 1 : st.prefix;
+    if (nc > 0 && !fallback)
       rank_candidates<F64>(w, unsigned(nc), take, tmin, st.done == 3, st.prefix, rsm, sh, wcnt, bins_out,
                            probs_out);
-    if (blockIdx.x == 0 && tid == 0) *n_found = int(take);
+    if (blockIdx.x == 0 && tid == 0 && !fallback) *n_found = int(take);
   } else if (tid == 0 && err) {
     atomicExch(err, 1);
   }
@@ -1858,6 +2286,8 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
       w.ctl[1] = 0ull;
       w.ctl[2] = 0ull;
       w.ctl[3] = 0ull;
+      w.ctl[4] = 0ull;
+      w.ctl[5] = 0ull;
     }
   }
 }
@@ -1905,14 +2335,19 @@ int select_resident_grid() {
     int dev = 0, sms = 152, p32 = 0, p64 = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(select_resident_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemMax);
-    cudaFuncSetAttribute(select_resident_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemMax);
-    cudaFuncSetAttribute(select_resident_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemMax);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p32, select_resident_kernel<false, false>, kRThreads, kRSmemMax);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p64, select_resident_kernel<true, false>, kRThreads, kRSmemMax);
+    cudaFuncSetAttribute(select_resident_kernel<false, NoSource>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemMax);
+    cudaFuncSetAttribute(select_resident_kernel<true, NoSource>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemMax);
+    cudaFuncSetAttribute(select_resident_kernel<false, TailArgs>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemMax);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p32, select_resident_kernel<false, NoSource>, kRThreads, kRSmemMax);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p64, select_resident_kernel<true, NoSource>, kRThreads, kRSmemMax);
     int pt = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pt, select_resident_kernel<false, true>, kRThreads, kRSmemMax);
-    int r = (p32 >= 1 && p64 >= 1 && pt >= 1) ? sms : 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pt, select_resident_kernel<false, TailArgs>, kRThreads, kRSmemMax);
+    int s32 = 0, s64 = 0;
+    cudaFuncSetAttribute(select_resident_kernel<false, StreamArgs>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemMax);
+    cudaFuncSetAttribute(select_resident_kernel<true, StreamArgs>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemMax);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s32, select_resident_kernel<false, StreamArgs>, kRThreads, kRSmemMax);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s64, select_resident_kernel<true, StreamArgs>, kRThreads, kRSmemMax);
+    int r = (p32 >= 1 && p64 >= 1 && pt >= 1 && s32 >= 1 && s64 >= 1) ? sms : 0;
     if (r > select_coop_grid()) r = select_coop_grid();   // tie counts live in the streaming part
     return r;
   }();
@@ -1966,11 +2401,11 @@ cudaError_t launch_select_resident(void* work, int grid, const void* x, int is_f
   ResWork w = resident_work(work);
   const int aligned = (reinterpret_cast<uintptr_t>(x) % 16) == 0;
   const unsigned long long kt = threshold_key(is_f64, threshold);
-  const TailArgs none{};
+  const NoSource none{};
   if (is_f64)
-    return launch_k(select_resident_kernel<true, false>, dim3(grid), dim3(kRThreads), smem, s, true, x, aligned, n,
+    return launch_k(select_resident_kernel<true, NoSource>, dim3(grid), dim3(kRThreads), smem, s, true, x, aligned, n,
                     per, kt, k, cap, w, bins_out, probs_out, n_found, err, none);
-  return launch_k(select_resident_kernel<false, false>, dim3(grid), dim3(kRThreads), smem, s, true, x, aligned, n,
+  return launch_k(select_resident_kernel<false, NoSource>, dim3(grid), dim3(kRThreads), smem, s, true, x, aligned, n,
                   per, kt, k, cap, w, bins_out, probs_out, n_found, err, none);
 }
 
@@ -2021,15 +2456,17 @@ cudaError_t launch_select_tail(void* work, int grid, const TailArgs& t, uint64_t
   const int cap = kMaxSort - k;
   ResWork w = resident_work(work);
   const unsigned long long kt = threshold_key(0, threshold);
-  return launch_k(select_resident_kernel<false, true>, dim3(grid), dim3(kRThreads), smem, s, true,
+  return launch_k(select_resident_kernel<false, TailArgs>, dim3(grid), dim3(kRThreads), smem, s, true,
                   static_cast<const void*>(nullptr), 0, n, per, kt, k, cap, w, bins_out, probs_out, n_found, err, ta);
 }
 
-cudaError_t launch_select_coop(void* work, int grid, const void* x, int is_f64, uint64_t n, int k, double threshold,
-                               unsigned long long* bins_out, double* probs_out, int* n_found, int* err,
-                               cudaStream_t s) {
-  if (k < 1 || k > kSelectMaxK) return cudaErrorInvalidValue;
-  const int cap = (k > 512 ? k : 512) < kMaxSort - k ? (k > 512 ? k : 512) : kMaxSort - k;
+namespace {
+// Bucket size at which the radix passes over the input stop.
+int coop_bucket_cap(int k) {
+  return (k > 512 ? k : 512) < kMaxSort - k ? (k > 512 ? k : 512) : kMaxSort - k;
+}
+// The streaming radix passes' part of the shared selection workspace.
+CoopWork coop_work(void* work) {
   char* p = static_cast<char*>(work);
   CoopWork w;
   w.ctl = reinterpret_cast<unsigned long long*>(p);
@@ -2043,6 +2480,50 @@ cudaError_t launch_select_coop(void* work, int grid, const void* x, int is_f64, 
   w.rank = reinterpret_cast<unsigned*>(p);
   p += sizeof(unsigned) * kMaxSort;
   w.tie_count = reinterpret_cast<unsigned*>(p);
+  return w;
+}
+}  // namespace
+
+cudaError_t launch_select_stream(void* work, int grid, const void* x, int is_f64, uint64_t n, int k,
+                                 double threshold, unsigned long long* bins_out, double* probs_out, int* n_found,
+                                 int* err, cudaStream_t s) {
+  if (k < 1 || k > kSelectMaxK || grid <= 0 || n < 1 || n > kStreamMost) return cudaErrorInvalidValue;
+  uint64_t per = (n + uint64_t(grid) - 1) / uint64_t(grid);
+  per = (per + 3) & ~uint64_t(3);
+  StreamArgs S{};
+  S.buf = unsigned(kRSmemMax - kRHistBytes - kRing * kRThreads * 16) / 8u;   // key word and bin per kept value
+  static_assert((kRSmemMax - kRHistBytes - kRing * kRThreads * 16) % 128 == 0, "16-byte slots");
+  S.coop = coop_work(work);
+  S.coop_cap = coop_bucket_cap(k);
+  if (n >= kFilterAllBelow) {
+    // tau: a few times k values above it, from kSampleAbove sampled values at
+    // least (n / 512 values kept then)
+    const uint64_t c = n >> 26;
+    S.chunks = unsigned(c < kSampleChunks ? kSampleChunks : (c > kSampleChunksMost ? kSampleChunksMost : c));
+    const uint64_t most = uint64_t(S.chunks) * kRThreads;
+    S.strata = unsigned(n / kSampleSpan < most ? n / kSampleSpan : most);
+    S.span = n / S.strata;
+    const uint64_t j = (4u * uint64_t(k > 2048 ? k : 2048)) * (uint64_t(kVec) * S.strata) / n;
+    S.j = unsigned(j < kSampleAbove ? kSampleAbove : (j > kSampleAboveMost ? kSampleAboveMost : j));
+  }
+  const int cap = kMaxSort - k;
+  ResWork w = resident_work(work);
+  const int aligned = (reinterpret_cast<uintptr_t>(x) % 16) == 0;
+  const unsigned long long kt = threshold_key(is_f64, threshold);
+  const size_t smem = kRSmemMax;
+  if (is_f64)
+    return launch_k(select_resident_kernel<true, StreamArgs>, dim3(grid), dim3(kRThreads), smem, s, true, x, aligned,
+                    n, per, kt, k, cap, w, bins_out, probs_out, n_found, err, S);
+  return launch_k(select_resident_kernel<false, StreamArgs>, dim3(grid), dim3(kRThreads), smem, s, true, x, aligned, n,
+                  per, kt, k, cap, w, bins_out, probs_out, n_found, err, S);
+}
+
+cudaError_t launch_select_coop(void* work, int grid, const void* x, int is_f64, uint64_t n, int k, double threshold,
+                               unsigned long long* bins_out, double* probs_out, int* n_found, int* err,
+                               cudaStream_t s) {
+  if (k < 1 || k > kSelectMaxK) return cudaErrorInvalidValue;
+  const int cap = coop_bucket_cap(k);
+  const CoopWork w = coop_work(work);
   const int aligned = (reinterpret_cast<uintptr_t>(x) % 16) == 0;
   const unsigned long long kt = threshold_key(is_f64, threshold);
   if (is_f64)
