@@ -1752,6 +1752,7 @@ SQC_API sqc_status sqc_create(sqc_ctx** out, int device, const sqc_config* cfg) 
   DeviceGuard g(device);
   e = select_configure();
   if (e == cudaSuccess) e = attr_configure();
+  if (e == cudaSuccess) e = gemm_simt_configure();
   if (e == cudaSuccess) e = gemm_tc_configure();
   if (e == cudaSuccess) e = batch_configure();
   if (e != cudaSuccess) return fail(nullptr, SQC_ECUDA, std::string("kernel setup: ") + cudaGetErrorString(e));

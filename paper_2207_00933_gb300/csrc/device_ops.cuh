@@ -1,6 +1,8 @@
 // Device-side bodies shared by the per-step kernels and the persistent
 // batched kernel: one merge CTA-block and one SIMT contraction tile.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace sqc {
@@ -68,6 +70,46 @@ template <bool CG>
 __device__ __forceinline__ float ld_operand(const float* p) {
   if constexpr (CG) return __ldcg(p);
   else return __ldg(p);
+}
+
+// A thread's TM x TN FP32 outputs (first row row0, first column c0), scaled and
+// written through the layout maps; returns their FP32 sum.
+template <int TM, int TN>
+__device__ __forceinline__ float store_tile_f32(const GemmArgs& a, const float (&acc)[TM][TN], int64_t row0,
+                                                int64_t c0, float alpha_f, void* Cout) {
+  float sum_f = 0.f;
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int64_t row = row0 + i;
+    if (row >= a.M) continue;
+    const uint64_t rbase = a.rowmap[row];
+    if (a.vec4 && (TN % 4) == 0 && c0 + TN <= a.N) {
+#pragma unroll
+      for (int j = 0; j + 3 < TN; j += 4) {
+        float4 q;
+        q.x = acc[i][j] * alpha_f; q.y = acc[i][j + 1] * alpha_f;
+        q.z = acc[i][j + 2] * alpha_f; q.w = acc[i][j + 3] * alpha_f;
+        sum_f += (q.x + q.y) + (q.z + q.w);
+        float4* dst = reinterpret_cast<float4*>(static_cast<float*>(Cout) + rbase + a.colmap[c0 + j]);
+        if (a.accumulate) {
+          const float4 o = *dst;
+          q.x += o.x; q.y += o.y; q.z += o.z; q.w += o.w;
+        }
+        *dst = q;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int64_t col = c0 + j;
+        if (col >= a.N) continue;
+        const float v = acc[i][j] * alpha_f;
+        sum_f += v;
+        float* dst = static_cast<float*>(Cout) + rbase + a.colmap[col];
+        *dst = a.accumulate ? *dst + v : v;
+      }
+    }
+  }
+  return sum_f;
 }
 
 // One BM x BN tile (origin m0, n0) of C = A B^T (Section 6.1) on NT threads
@@ -176,6 +218,8 @@ __device__ __forceinline__ double gemm_tile(const GemmArgs& a, int64_t m0, int64
 
   // FP32 outputs are scaled and summed in FP32; only FP64 outputs use the
   // FP64 pipe per element
+  if constexpr (!CHUNKED)
+    if (a.kind == OUT_F32) return double(store_tile_f32<TM, TN>(a, acc, m0 + ty * TM, n0 + tx * TN, alpha_f, Cout));
   float sum_f = 0.f;
   double sum_d = 0.0;
 #pragma unroll
@@ -184,53 +228,153 @@ __device__ __forceinline__ double gemm_tile(const GemmArgs& a, int64_t m0, int64
     if (row >= a.M) continue;
     const uint64_t rbase = a.rowmap[row];
     const int64_t c0 = n0 + tx * TN;
-    if (!CHUNKED && a.kind == OUT_F32) {
-      if (a.vec4 && (TN % 4) == 0 && c0 + TN <= a.N) {
 #pragma unroll
-        for (int j = 0; j < TN; j += 4) {
-          float4 q;
-          q.x = acc[i][j] * alpha_f; q.y = acc[i][j + 1] * alpha_f;
-          q.z = acc[i][j + 2] * alpha_f; q.w = acc[i][j + 3] * alpha_f;
-          sum_f += (q.x + q.y) + (q.z + q.w);
-          float4* dst = reinterpret_cast<float4*>(static_cast<float*>(Cout) + rbase + a.colmap[c0 + j]);
-          if (a.accumulate) {
-            const float4 o = *dst;
-            q.x += o.x; q.y += o.y; q.z += o.z; q.w += o.w;
-          }
-          *dst = q;
-        }
+    for (int j = 0; j < TN; ++j) {
+      const int64_t col = c0 + j;
+      if (col >= a.N) continue;
+      double v;
+      if constexpr (CHUNKED) v = acc64[i][j]; else v = f2d(acc[i][j] * alpha_f);
+      if (a.kind == OUT_F64) sum_d += v; else sum_f += float(v);
+      if (a.accumulate && a.kind == OUT_F64) {
+        double* dst = static_cast<double*>(Cout) + rbase + a.colmap[col];
+        *dst += v;                          // slices add up in FP64
+      } else if (a.accumulate && a.kind == OUT_F32) {
+        float* dst = static_cast<float*>(Cout) + rbase + a.colmap[col];
+        *dst += float(v);
       } else {
-#pragma unroll
-        for (int j = 0; j < TN; ++j) {
-          const int64_t col = c0 + j;
-          if (col >= a.N) continue;
-          const float v = acc[i][j] * alpha_f;
-          sum_f += v;
-          float* dst = static_cast<float*>(Cout) + rbase + a.colmap[col];
-          *dst = a.accumulate ? *dst + v : v;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < TN; ++j) {
-        const int64_t col = c0 + j;
-        if (col >= a.N) continue;
-        double v;
-        if constexpr (CHUNKED) v = acc64[i][j]; else v = f2d(acc[i][j] * alpha_f);
-        if (a.kind == OUT_F64) sum_d += v; else sum_f += float(v);
-        if (a.accumulate && a.kind == OUT_F64) {
-          double* dst = static_cast<double*>(Cout) + rbase + a.colmap[col];
-          *dst += v;                          // slices add up in FP64
-        } else if (a.accumulate && a.kind == OUT_F32) {
-          float* dst = static_cast<float*>(Cout) + rbase + a.colmap[col];
-          *dst += float(v);
-        } else {
-          store_out(Cout, a.kind, a.plane_stride, rbase + a.colmap[col], v);
-        }
+        store_out(Cout, a.kind, a.plane_stride, rbase + a.colmap[col], v);
       }
     }
   }
   return sum_d + double(sum_f);
+}
+
+// Two FP32 multiply-adds in one instruction (each rounded as fmaf does).
+__device__ __forceinline__ void fma2(float2& d, float2 a, float2 b) {
+  unsigned long long& dd = reinterpret_cast<unsigned long long&>(d);
+  asm("fma.rn.f32x2 %0, %1, %2, %0;"
+      : "+l"(dd)
+      : "l"(reinterpret_cast<unsigned long long&>(a)), "l"(reinterpret_cast<unsigned long long&>(b)));
+}
+
+// The same tile of a long shared index (K a multiple of kPipeK, whole tiles:
+// M a multiple of BM, N of BN; FP32 output), for steps that are bound by the
+// FP32 units: the next stage's operands (16-byte loads) travel in registers,
+// A during the first half of the current stage and B during the second, into
+// the other shared-memory buffer (one CTA barrier per stage), and the
+// multiply-adds are issued two columns at a time.  k runs upwards as in
+// gemm_tile, so the values are the same bit for bit.  B's columns lie in
+// shared memory with the two float4 halves of a thread's 8 columns apart, so
+// that a warp's 16-byte reads do not collide.  128 threads with 8 x 8 outputs
+// each, three CTAs per SM.  (Measured and not kept: 16 x 8 outputs a thread,
+// two CTAs per SM, 1.4% faster at 4096 x 4096 x 256 and 11% slower at
+// 4096 x 2048 x 256; A doubled in shared memory to save the register moves,
+// 13% slower.)
+// 4096 x 4096 x 256: 178 us, 48 TFLOP/s of the 75 that packed multiply-adds
+// reach from registers (gemm_tile's unbuffered stages and scalar loads: 218
+// us); 4096 x 2048 x 256 131 -> 95 us, 4096 x 2048 x 64 47 -> 37 us.
+constexpr int kPipeK = 16;
+template <int BM, int BN>
+constexpr int gemm_pipe_smem_floats() {
+  return 2 * kPipeK * (BM + 4 + BN + 4);
+}
+constexpr int kPipeThreads = 128;
+template <int BM, int BN, int TM, int TN, bool CG = false>
+__device__ __forceinline__ double gemm_tile_pipe(const GemmArgs& a, int64_t m0, int64_t n0, float* smem,
+                                                 void* Cout) {
+  constexpr int NT = kPipeThreads, TX = BN / TN;
+  static_assert((BM / TM) * TX == NT && TM % 8 == 0 && TN % 4 == 0 && TN <= 8, "tile shape");
+  constexpr int SA = BM + 4, SB = BN + 4, kStage = kPipeK * (SA + SB);
+  constexpr int kQ = kPipeK / 4;                     // float4 per row and stage
+  constexpr int LA = BM * kQ / NT, LB = BN * kQ / NT;
+  static_assert(LA * NT == BM * kQ && LB * NT == BN * kQ, "whole loads");
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const float* A = a.A + m0 * a.K;
+  const float* B = a.B + n0 * a.K;
+  auto ld4 = [](const float* p) -> float4 {
+    if constexpr (CG) return __ldcg(reinterpret_cast<const float4*>(p));
+    else return __ldg(reinterpret_cast<const float4*>(p));
+  };
+  // position of column c in a row of the B stage
+  auto bpos = [](int c) -> int { return TN == 8 ? ((c >> 2) & 1) * (BN / 2) + (c >> 3) * 4 + (c & 3) : c; };
+  constexpr int LR = LA > LB ? LA : LB;
+  float4 r[LR];                                      // one operand of the next stage on its way
+  auto fetch = [&](const float* P, auto cnt, int64_t k0) {
+#pragma unroll
+    for (int u = 0; u < cnt.value; ++u) {
+      const int i = tid + u * NT;
+      r[u] = ld4(P + int64_t(i / kQ) * a.K + k0 + 4 * (i % kQ));
+    }
+  };
+  auto put_a = [&](float* st) {
+#pragma unroll
+    for (int u = 0; u < LA; ++u) {
+      const int i = tid + u * NT;
+      float* p = st + 4 * (i % kQ) * SA + i / kQ;
+      p[0] = r[u].x; p[SA] = r[u].y; p[2 * SA] = r[u].z; p[3 * SA] = r[u].w;
+    }
+  };
+  auto put_b = [&](float* st) {
+#pragma unroll
+    for (int u = 0; u < LB; ++u) {
+      const int i = tid + u * NT;
+      float* p = st + kPipeK * SA + 4 * (i % kQ) * SB + bpos(i / kQ);
+      p[0] = r[u].x; p[SB] = r[u].y; p[2 * SB] = r[u].z; p[3 * SB] = r[u].w;
+    }
+  };
+  const std::integral_constant<int, LA> la{};
+  const std::integral_constant<int, LB> lb{};
+  float2 acc[TM][TN / 2];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN / 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  auto multiply = [&](const float* sa, const float* sb) {   // half a stage
+#pragma unroll
+    for (int kk = 0; kk < kPipeK / 2; ++kk) {
+      float4 af[TM / 4], bf[TN / 4];
+#pragma unroll
+      for (int i = 0; i < TM / 4; ++i) af[i] = *reinterpret_cast<const float4*>(sa + kk * SA + 4 * i);
+#pragma unroll
+      for (int j = 0; j < TN / 4; ++j) bf[j] = *reinterpret_cast<const float4*>(sb + kk * SB + j * (BN / 2));
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const float x = reinterpret_cast<const float*>(af)[i];
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], make_float2(x, x), reinterpret_cast<const float2*>(bf)[j]);
+      }
+    }
+  };
+  fetch(A, la, 0);
+  put_a(smem);
+  fetch(B, lb, 0);
+  put_b(smem);
+  __syncthreads();
+  int cur = 0;
+  for (int64_t k0 = 0; k0 < a.K; k0 += kPipeK) {
+    const bool more = k0 + kPipeK < a.K;
+    const float* st = smem + cur * kStage;
+    float* next = smem + (cur ^ 1) * kStage;
+    const float* sa = st + ty * TM;
+    const float* sb = st + kPipeK * SA + 4 * tx;
+    if (more) fetch(A, la, k0 + kPipeK);
+    multiply(sa, sb);
+    if (more) {
+      put_a(next);
+      fetch(B, lb, k0 + kPipeK);
+    }
+    multiply(sa + kPipeK / 2 * SA, sb + kPipeK / 2 * SB);
+    if (more) put_b(next);
+    __syncthreads();
+    cur ^= 1;
+  }
+  // (the probability check's FP32 groups: 8 rows, as gemm_tile's)
+  double sum = 0.0;
+#pragma unroll
+  for (int i = 0; i < TM; i += 8)
+    sum += double(store_tile_f32<8, TN>(a, reinterpret_cast<const float(&)[8][TN]>(acc[i]), m0 + ty * TM + i,
+                                        n0 + tx * TN, pow2_to_float(a.alpha), Cout));
+  return sum;
 }
 
 

@@ -37,6 +37,26 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(GemmArgs a) {
   if (a.partials) finish_total(mysum, a.partials, a.counter, a.total, red);
 }
 
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__(kPipeThreads, 3) gemm_pipe_kernel(GemmArgs a) {
+  pdl_wait();      // the previous kernel on the stream has completed
+  pdl_trigger();   // the next one may start launching
+  extern __shared__ __align__(16) float smem[];
+  __shared__ double red[kPipeThreads / 32];
+  const int tn_shift = __ffsll(a.N / BN) - 1;
+  const int64_t tile = blockIdx.x;
+  const int64_t m0 = (tile >> tn_shift) * BM;
+  const int64_t n0 = (tile & ((int64_t(1) << tn_shift) - 1)) * BN;
+  const double mysum = gemm_tile_pipe<BM, BN, TM, TN>(a, m0, n0, smem, a.C);
+  if (a.partials) finish_total(mysum, a.partials, a.counter, a.total, red);
+}
+
+template <int BM, int BN, int TM, int TN>
+cudaError_t launch_pipe(const GemmArgs& a, cudaStream_t s) {
+  return launch_k(gemm_pipe_kernel<BM, BN, TM, TN>, dim3(unsigned((a.M / BM) * (a.N / BN))), dim3(kPipeThreads),
+                  sizeof(float) * gemm_pipe_smem_floats<BM, BN>(), s, false, a);
+}
+
 template <int BM, int BN, int TM, int TN, bool CH, int BK = 16>
 cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
   const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
@@ -56,12 +76,24 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
 
 }  // namespace
 
+cudaError_t gemm_simt_configure() {
+  return cudaFuncSetAttribute(gemm_pipe_kernel<128, 64, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              int(sizeof(float)) * gemm_pipe_smem_floats<128, 64>());
+}
+
 cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaErrorInvalidValue;
   const bool chunked = a.chunk > 0;
   const bool wide = !chunked && a.kind == OUT_F32;
   auto tiles = [&](int bm, int bn) { return ((a.M + bm - 1) / bm) * ((a.N + bn - 1) / bn); };
   const int64_t want = 152;   // at least one full wave of CTAs
+  // the pipelined form: whole tiles (M, N, K are powers of two) for every SM,
+  // two stages or more -- with a single stage there is nothing to overlap --
+  // and 16-byte aligned operands
+  const int64_t pipe_tiles = (a.M / 128) * (a.N / 64);
+  if (wide && a.K >= 2 * kPipeK && pipe_tiles >= want && pipe_tiles <= 0x7fffffff &&
+      ((reinterpret_cast<uintptr_t>(a.A) | reinterpret_cast<uintptr_t>(a.B)) & 15) == 0)
+    return launch_pipe<128, 64, 8, 8>(a, s);
   if (wide && tiles(128, 128) >= want) return launch_cfg<128, 128, 8, 8, false>(a, s);
   if (!wide && tiles(128, 64) >= want) {
     if (chunked) return launch_cfg<128, 64, 8, 4, true>(a, s);

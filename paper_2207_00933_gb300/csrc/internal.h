@@ -166,6 +166,7 @@ struct GemmArgs {
   double* total;
 };
 cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t s);
+cudaError_t gemm_simt_configure();   // one-time kernel attributes (dynamic shared memory)
 
 // ---- contraction step, split-BF16 on tcgen05 ---------------------------------
 struct GemmTcArgs {
