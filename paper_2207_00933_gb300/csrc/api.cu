@@ -34,6 +34,9 @@ thread_local std::string g_create_error;
 constexpr int kBinBase = 1 << 16;   // layout codes: edge bit = 2*eid + (hi?1:0); bin bit = kBinBase + position
 constexpr int kMaxK = 16;           // cut edges per subcircuit
 constexpr int kMaxSub = 64;
+// Most outputs of a query merged by one warp each in small CTAs
+// (launch_merge_long): beyond, the plain kernel has warps enough.
+constexpr int64_t kMergeLongMost = 8192;
 
 struct Circuit {
   int n_qubits = 0, nC = 0, K = 0;
@@ -103,6 +106,8 @@ struct Plan {
   std::vector<MergeDesc> merge_host;
   MergeDesc* merge_dev = nullptr;
   int64_t merge_blocks = 0;
+  bool merge_tiled = false;
+  int64_t merge_long = 0;        // > 0: merged by launch_merge_long (outputs)
   void* work = nullptr;
   size_t work_bytes = 0;
   double* partials = nullptr;
@@ -1197,7 +1202,8 @@ sqc_status finalize_plan(sqc_ctx* ctx, Plan* P) {
     P->steps[s].rowmap = maps_dev + D.step_map_off[s].first;
     P->steps[s].colmap = maps_dev + D.step_map_off[s].second;
   }
-  int64_t blocks = 0;
+  int64_t blocks = 0, long_outputs = 0;
+  bool all_long = true, any_tiled = false;
   for (int i = 0; i < nC; ++i) {
     MergeDesc& d = P->merge_host[i];
     d.rowmap = maps_dev + D.merge_map_off[i].first;
@@ -1207,12 +1213,33 @@ sqc_status finalize_plan(sqc_ctx* ctx, Plan* P) {
     d.plane_stride = P->tensors[i].plane_stride;
     d.rowsel = D.has_rowsel[i] ? maps_dev + D.rowsel_off[i] : nullptr;
     d.row_add = 0;
+    // Rows that are consecutive in the destination (its lowest address bits
+    // are row bits) and bins at least a sector apart, one thread per output:
+    // turned in shared memory.  From 2^18 outputs, where the 2048-output
+    // tiles still reach most SMs.
+    const std::vector<int>& lay = P->tensors[i].layout;
+    const int rowbits = ilog2(d.rows);
+    {
+      std::vector<std::pair<uint64_t, int>> at;      // (destination bit, row bit)
+      const uint64_t* rm = D.maps.data() + D.merge_map_off[i].first;
+      for (int j = 0; j < rowbits; ++j) at.push_back({rm[size_t(1) << j], j});
+      std::sort(at.begin(), at.end());
+      const int tr = std::min(rowbits, 5);
+      bool contiguous = tr >= 3;
+      for (int j = 0; j < tr && contiguous; ++j) contiguous = at[j].first == (uint64_t(1) << j);
+      for (int j = 0; j < rowbits; ++j) d.rowbit[j] = static_cast<unsigned char>(at[j].second);
+      d.tiled = contiguous && d.lanes == 1 && d.a >= 6 && (d.rows << d.a) >= (int64_t(1) << 18) &&
+                int(lay.size()) > 0 && i != P->final_tensor;
+    }
     d.block_begin = blocks;
-    const int64_t outs = d.rows << d.a;
-    const int64_t per = 256 / d.lanes;
-    blocks += (outs + per - 1) / per;
+    blocks += merge_blocks_of(d);
+    long_outputs += d.rows << d.a;
+    all_long = all_long && merge_is_long(d);
+    any_tiled = any_tiled || d.tiled;
   }
   P->merge_blocks = blocks;
+  P->merge_tiled = any_tiled;
+  P->merge_long = all_long && long_outputs <= kMergeLongMost ? long_outputs : 0;
   cudaError_t e = upload(ctx, maps_dev, D.maps.data(), sizeof(uint64_t) * D.maps.size());
   if (e == cudaSuccess && nC > 0) {
     // one descriptor set per slice: slice sigma fixes sliced edge j's digit
@@ -1435,9 +1462,7 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
     for (int i = 0; i < c.nC; ++i) {
       const int di = int(mdescs.size());
       mdescs.push_back(P.merge_host[i]);
-      const MergeDesc& d = P.merge_host[i];
-      const int64_t per = 256 / d.lanes;
-      const int64_t nblk = ((d.rows << d.a) + per - 1) / per;
+      const int64_t nblk = merge_blocks_of(P.merge_host[i]);
       for (int64_t b = 0; b < nblk; ++b) items.push_back({{kItemMerge, di, b, -1, -1, slot[i]}, 0, 0});
       expected[slot[i]] = unsigned(nblk);
     }
@@ -2198,7 +2223,8 @@ sqc_status reconstruct_stages(sqc_ctx* ctx, sqc_query_id qid, sqc_precision prec
       }
       return SQC_OK;
     }
-    CK(launch_merge_blocks(descs, nd, P.merge_blocks, s));
+    if (P.merge_long > 0) CK(launch_merge_long(descs, nd, P.merge_long, s));
+    else CK(launch_merge_blocks(descs, nd, P.merge_blocks, P.merge_tiled, s));
     ctx->launches += 1;
     return SQC_OK;
   };

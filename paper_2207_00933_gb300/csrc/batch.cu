@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(kOpThreads, 2) batch_kernel(BatchLaunch L) {
     __syncthreads();
     if (!skip) {
       if (item.type == kItemMerge) {
-        merge_block(md, item.tile);
+        if (md.tiled) merge_tile(md, item.tile, smem);
+        else merge_block(md, item.tile);
       } else {
         const BatchStep& st = L.steps[item.idx];
         // a single-query launch names its output and probability sum per

@@ -9,6 +9,180 @@ namespace sqc {
 
 constexpr int kOpThreads = 256;
 
+// One lane's share of the sum over output (row of A, bin b) of descriptor d:
+// every lanes-th 16-byte word of the run (or every lanes-th value).
+__device__ __forceinline__ float merge_sum(const MergeDesc& d, const float* row, uint32_t b, uint32_t lane,
+                                           uint32_t lanes) {
+  float acc = 0.f;
+  const uint32_t run = 1u << d.m;
+  if (d.fast) {
+    const float* src = row + (d.zoom_val | (b << d.m));
+    if (run >= 4u * lanes) {
+      // four independent 16-byte loads in flight per lane and round
+      const float4* s4 = reinterpret_cast<const float4*>(src);
+      const uint32_t nv = run / 4;
+      uint32_t r = lane;
+      for (; r + 3u * lanes < nv; r += 4u * lanes) {
+        const float4 q0 = __ldg(s4 + r), q1 = __ldg(s4 + r + lanes);
+        const float4 q2 = __ldg(s4 + r + 2u * lanes), q3 = __ldg(s4 + r + 3u * lanes);
+        acc += (((q0.x + q0.y) + (q0.z + q0.w)) + ((q1.x + q1.y) + (q1.z + q1.w))) +
+               (((q2.x + q2.y) + (q2.z + q2.w)) + ((q3.x + q3.y) + (q3.z + q3.w)));
+      }
+      for (; r < nv; r += lanes) {
+        const float4 q = __ldg(s4 + r);
+        acc += (q.x + q.y) + (q.z + q.w);
+      }
+    } else {
+      for (uint32_t r = lane; r < run; r += lanes) acc += __ldg(src + r);
+    }
+  } else {
+    const uint32_t xb = deposit(b, d.act_mask) | d.zoom_val;
+    for (uint32_t r = lane; r < run; r += lanes) acc += __ldg(row + (xb | deposit(r, d.mer_mask)));
+  }
+  return acc;
+}
+
+// Row of A that descriptor row e reads.
+__device__ __forceinline__ const float* merge_row(const MergeDesc& d, int64_t e) {
+  const int64_t er = d.rowsel ? int64_t(d.rowsel[e]) + d.row_add : e;
+  return d.A + (er << d.n);
+}
+
+// The sums of a turned tile (merge_tile) over runs of 2^MB states: 2^MB / 4
+// lanes per output, one 16-byte word each, so that a warp reads whole lines,
+// and U rows' loads in flight per thread.  The additions are merge_sum's (one
+// lane), in its order.
+template <int MB, int U>
+__device__ __forceinline__ void merge_tile_rows(const MergeDesc& d, const float* const* rows, uint32_t bin0, int nr,
+                                                float alpha, float* tile) {
+  constexpr int SB = kMergeTileBins + 1, L = MB > 2 ? 1 << (MB - 2) : 1, RP = 4 / L;
+  const int sub = threadIdx.x & (L - 1), bin = (threadIdx.x / L) & 63, rg = threadIdx.x / (64 * L);
+  const uint32_t at = (d.zoom_val | ((bin0 + bin) << MB)) + 4 * sub;
+  for (int r0 = rg; r0 < nr; r0 += RP * U) {
+    float4 w[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      w[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      const int r = r0 + RP * u;
+      if (r >= nr) continue;
+      const float* src = rows[r] + at;
+      if constexpr (MB == 0) {
+        w[u].x = __ldg(src);
+      } else if constexpr (MB == 1) {
+        const float2 t = __ldg(reinterpret_cast<const float2*>(src));
+        w[u].x = t.x; w[u].y = t.y;
+      } else {
+        w[u] = __ldg(reinterpret_cast<const float4*>(src));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      float acc = 0.f;
+      if constexpr (MB == 0) {
+        acc += w[u].x;
+      } else if constexpr (MB == 1) {
+        acc += w[u].x;
+        acc += w[u].y;
+      } else {
+        float t = (w[u].x + w[u].y) + (w[u].z + w[u].w);
+        if constexpr (MB == 4) {                     // ((0) + (1)) + ((2) + (3))
+          t += __shfl_xor_sync(0xffffffffu, t, 1);
+          t += __shfl_xor_sync(0xffffffffu, t, 2);
+          acc += t;
+        } else if constexpr (MB == 3) {              // (0) + (1)
+          const float o = __shfl_xor_sync(0xffffffffu, t, 1);
+          acc += t;
+          acc += o;
+        } else {
+          acc += t;
+        }
+      }
+      const int r = r0 + RP * u;
+      if (sub == 0 && r < nr) tile[r * SB + bin] = acc * alpha;
+    }
+  }
+}
+
+// One tile of up to 32 rows x 64 bins of a descriptor whose rows are
+// consecutive in the destination while its bins lie a whole operand row
+// apart (a contraction operand: the shared cut edges innermost).  Bins are
+// read along A's rows, the sums turned in shared memory, and consecutive rows
+// written as 16-byte words: written as they are read, every 4-byte (BF16: 2-
+// byte) value would touch a sector of its own.  smem: kMergeTileFloats.
+// Bound: HBM.  256 rows x 4096 bins of one value and of 16 (71 MB): into FP32
+// operands 29 -> 21 us, into BF16 planes 62 -> 23 us; 64 rows x 4096 bins of
+// two and of 16 values, FP32, 12.9 -> 10.3 us.
+constexpr int kMergeTileFloats = kMergeTileRows * (kMergeTileBins + 1) + 2 * kMergeTileRows + 2 * kMergeTileBins;
+__device__ __forceinline__ void merge_tile(const MergeDesc& d, int64_t blk, float* smem) {
+  constexpr int SB = kMergeTileBins + 1;
+  const float** rows = reinterpret_cast<const float**>(smem);              // [kMergeTileRows]
+  uint64_t* cols = reinterpret_cast<uint64_t*>(smem + 2 * kMergeTileRows);  // [kMergeTileBins]
+  float* tile = smem + 2 * kMergeTileRows + 2 * kMergeTileBins;
+  const int lr = d.rows < kMergeTileRows ? __ffsll(d.rows) - 1 : 5;      // log2 of the tile's rows
+  const int nr = 1 << lr;
+  const int64_t bt = blk & ((int64_t(1) << (d.a - 6)) - 1), rt = blk >> (d.a - 6);
+  const uint32_t bin0 = uint32_t(bt) * kMergeTileBins;
+  __shared__ uint64_t base;
+  const int tid = threadIdx.x;
+  if (tid < nr) {
+    const int nbits = __ffsll(d.rows) - 1;
+    const int64_t r = (rt << lr) + tid;                                  // r-th row in destination order
+    int64_t e = 0;
+    for (int j = 0; j < nbits; ++j) e |= ((r >> j) & 1) << d.rowbit[j];
+    rows[tid] = merge_row(d, e);
+    if (tid == 0) base = d.rowmap[e];
+  } else if (tid >= 64 && tid < 64 + kMergeTileBins) {
+    cols[tid - 64] = d.colmap[bin0 + tid - 64];
+  }
+  __syncthreads();
+  const float alpha = pow2_to_float(d.alpha);
+  if (d.fast && d.m <= 4) {
+    switch (d.m) {
+      case 0: merge_tile_rows<0, 8>(d, rows, bin0, nr, alpha, tile); break;
+      case 1: merge_tile_rows<1, 8>(d, rows, bin0, nr, alpha, tile); break;
+      case 2: merge_tile_rows<2, 8>(d, rows, bin0, nr, alpha, tile); break;
+      case 3: merge_tile_rows<3, 8>(d, rows, bin0, nr, alpha, tile); break;
+      default: merge_tile_rows<4, 8>(d, rows, bin0, nr, alpha, tile); break;
+    }
+  } else {
+    for (int r = tid >> 6; r < nr; r += 4) tile[r * SB + (tid & 63)] = merge_sum(d, rows[r], bin0 + (tid & 63), 0, 1) * alpha;
+  }
+  __syncthreads();
+  if (d.kind == OUT_F32) {
+    for (int i = tid; i < (nr * kMergeTileBins) >> 2; i += 256) {
+      const int r = 4 * (i & ((nr >> 2) - 1)), c = i >> (lr - 2);
+      const float* t = tile + r * SB + c;
+      float* p = static_cast<float*>(d.dst) + base + cols[c] + r;
+      *reinterpret_cast<float4*>(p) = make_float4(t[0], t[SB], t[2 * SB], t[3 * SB]);
+    }
+  } else {                                           // OUT_BF16X3
+    for (int i = tid; i < (nr * kMergeTileBins) >> 3; i += 256) {
+      const int r = 8 * (i & ((nr >> 3) - 1)), c = i >> (lr - 3);
+      const float* t = tile + r * SB + c;
+      uint32_t w[3][4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        __nv_bfloat16 h[2][3];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {                // as store_out_f splits a value
+          const float f = t[(2 * q + u) * SB];
+          h[u][0] = __float2bfloat16_rn(f);
+          const float r1 = f - __bfloat162float(h[u][0]);
+          h[u][1] = __float2bfloat16_rn(r1);
+          h[u][2] = __float2bfloat16_rn(r1 - __bfloat162float(h[u][1]));
+        }
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+          w[p][q] = uint32_t(__bfloat16_as_ushort(h[0][p])) | uint32_t(__bfloat16_as_ushort(h[1][p])) << 16;
+      }
+      __nv_bfloat16* o = static_cast<__nv_bfloat16*>(d.dst) + base + cols[c] + r;
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        *reinterpret_cast<uint4*>(o + p * d.plane_stride) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+    }
+  }
+}
+
 // One CTA-block of the merge of descriptor d (Section 4, Algorithm 2):
 // blk is the block index relative to the descriptor's first block.
 __device__ __forceinline__ void merge_block(const MergeDesc& d, int64_t blk) {
@@ -19,37 +193,7 @@ __device__ __forceinline__ void merge_block(const MergeDesc& d, int64_t blk) {
   const int64_t total = d.rows << d.a;
   const bool valid = o < total;
   float acc = 0.f;
-  if (valid) {
-    const int64_t e = o >> d.a;
-    const uint32_t b = uint32_t(o & ((int64_t(1) << d.a) - 1));
-    const int64_t er = d.rowsel ? int64_t(d.rowsel[e]) + d.row_add : e;
-    const float* row = d.A + (er << d.n);
-    const uint32_t run = 1u << d.m;
-    if (d.fast) {
-      const float* src = row + (d.zoom_val | (b << d.m));
-      if (run >= 4u * lanes) {
-        // four independent 16-byte loads in flight per lane and round
-        const float4* s4 = reinterpret_cast<const float4*>(src);
-        const uint32_t nv = run / 4;
-        uint32_t r = lane;
-        for (; r + 3u * lanes < nv; r += 4u * lanes) {
-          const float4 q0 = __ldg(s4 + r), q1 = __ldg(s4 + r + lanes);
-          const float4 q2 = __ldg(s4 + r + 2u * lanes), q3 = __ldg(s4 + r + 3u * lanes);
-          acc += (((q0.x + q0.y) + (q0.z + q0.w)) + ((q1.x + q1.y) + (q1.z + q1.w))) +
-                 (((q2.x + q2.y) + (q2.z + q2.w)) + ((q3.x + q3.y) + (q3.z + q3.w)));
-        }
-        for (; r < nv; r += lanes) {
-          const float4 q = __ldg(s4 + r);
-          acc += (q.x + q.y) + (q.z + q.w);
-        }
-      } else {
-        for (uint32_t r = lane; r < run; r += lanes) acc += __ldg(src + r);
-      }
-    } else {
-      const uint32_t xb = deposit(b, d.act_mask) | d.zoom_val;
-      for (uint32_t r = lane; r < run; r += lanes) acc += __ldg(row + (xb | deposit(r, d.mer_mask)));
-    }
-  }
+  if (valid) acc = merge_sum(d, merge_row(d, o >> d.a), uint32_t(o & ((int64_t(1) << d.a) - 1)), lane, lanes);
   for (int off = lanes >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
   if (valid && lane == 0) {
     const int64_t e = o >> d.a;

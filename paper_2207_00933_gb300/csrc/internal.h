@@ -126,6 +126,8 @@ struct MergeDesc {
   int a, m;                               // active / merged bit counts
   int fast;                               // mer_mask == low m bits, act_mask == next a bits
   int lanes;                              // threads cooperating on one output (1..32, pow2)
+  int tiled;                              // outputs transposed through shared memory (merge_tile)
+  unsigned char rowbit[32];               // bit of the row index at the j-th lowest destination position
   const uint64_t* rowmap;                 // [rows]
   const uint64_t* colmap;                 // [2^a]
   void* dst;
@@ -139,8 +141,25 @@ struct MergeDesc {
   int64_t row_add;
 };
 constexpr int kMaxMerge = 64;
-// descs: device array of n descriptors; total_blocks = CTAs over all of them
-cudaError_t launch_merge_blocks(const MergeDesc* descs, int n, int64_t total_blocks, cudaStream_t s);
+constexpr int kMergeTileBins = 64;        // bins of a transposed tile
+constexpr int kMergeTileRows = 32;        // and rows at most
+// CTA blocks (256 threads) of one descriptor
+inline int64_t merge_blocks_of(const MergeDesc& d) {
+  if (d.tiled) {
+    const int64_t tr = d.rows < kMergeTileRows ? d.rows : kMergeTileRows;
+    return (d.rows / tr) << (d.a - 6);
+  }
+  const int64_t per = 256 / d.lanes;
+  return ((d.rows << d.a) + per - 1) / per;
+}
+// Whether merge_long_kernel can take a descriptor: contiguous runs of a warp's
+// rounds (512 states) at least.
+inline bool merge_is_long(const MergeDesc& d) { return d.fast && d.lanes == 32 && d.m >= 9; }
+// descs: device array of n descriptors; total_blocks = CTAs over all of them;
+// tiled: some descriptor is
+cudaError_t launch_merge_blocks(const MergeDesc* descs, int n, int64_t total_blocks, bool tiled, cudaStream_t s);
+// The same for descriptors that are all merge_is_long, total_outputs of them
+cudaError_t launch_merge_long(const MergeDesc* descs, int n, int64_t total_outputs, cudaStream_t s);
 // Merge pyramid of one subcircuit (A: [V][2^n]): level m = 1..n at
 // pyr + V (2^n - 2^(n-m+1)), [V][2^(n-m)], level m = pairwise sums of level
 // m-1 (level 0 = A).  One launch per kPyramidLevelsPerPass levels.

@@ -12,11 +12,19 @@ from synthetic.circuits import chain_line_circuit
 pytestmark = pytest.mark.gpu
 
 
-def _chain(seed, widths, cuts, most=2):
+def _chain(seed, widths, cuts, most=2, ones=None):
+    """A chain with outputs in 0..most, or with `ones` ones per variant."""
     c = chain_line_circuit(seed, widths, cuts, 1)
     rng = np.random.default_rng(seed)
-    probs = [rng.integers(0, most + 1, (4 ** len(c.incident[i]), 1 << c.width(i))).astype(np.float32)
-             for i in range(c.n_subcircuits)]
+    probs = []
+    for i in range(c.n_subcircuits):
+        shape = (4 ** len(c.incident[i]), 1 << c.width(i))
+        if ones is None:
+            p = rng.integers(0, most + 1, shape)
+        else:
+            p = np.zeros(shape)
+            p[np.arange(shape[0])[:, None], rng.integers(0, shape[1], (shape[0], ones))] = 1
+        probs.append(p.astype(np.float32))
     return c, probs
 
 
@@ -36,7 +44,10 @@ def _run(c, probs, roles, precision="fp32", out="float32", **cfg):
 
 def _check(c, probs, roles, **kw):
     g = O.Graph.from_arrays(c.n_qubits, *c.graph_arrays())
-    ref = O.reconstruct(g, [p.astype(np.float64) for p in probs], roles)
+    T = O.subcircuit_tensors(g, [p.astype(np.float64) for p in probs], roles)
+    # the premise: no partial sum of the contraction reaches 2^24 (the 2^-K is exact)
+    assert O.reconstruct_pairwise(g, [np.abs(t) for t in T], roles).max() * 2.0 ** c.n_edges < 2 ** 24
+    ref = O.reconstruct_pairwise(g, T, roles)
     got, tot, steps = _run(c, probs, roles, **kw)
     assert np.array_equal(got, ref), (steps, np.abs(got - ref).max())
     assert abs(tot - ref.sum()) <= 1e-6 * np.abs(ref).sum()
@@ -54,3 +65,44 @@ def test_pipelined_step(widths, cut, active, shape):
     c, probs = _chain(sum(widths) + cut, widths, [cut], most=1)
     steps = _check(c, probs, W.lowest_active_roles(c, active))
     assert tuple(sorted(steps[-1][:2])) == tuple(sorted(shape[:2])) and steps[-1][2] == shape[2]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "split_bf16"])
+@pytest.mark.parametrize("widths,cut,active", [
+    ([14, 13], 2, [12, 13]),          # 16 rows: 2^16 and 2^17 outputs, value by value
+    ([16, 14], 2, [14, 14]),          # 16 rows, 2^18 outputs: half-height tiles
+    ([15, 14], 3, [12, 12]),          # 64 rows, one and four states per bin
+    ([14, 14], 4, [10, 10]),          # 256 rows, 1 and 16 states per bin
+    ([14, 13], 4, [9, 10]),           # 2 and 8 states per bin; the first below the tiles' size
+])
+def test_turned_merge(widths, cut, active, precision):
+    c, probs = _chain(sum(widths) + cut, widths, [cut], most=1)
+    _check(c, probs, W.lowest_active_roles(c, active), precision=precision)
+
+
+def test_turned_merge_other_roles():
+    """Bins that are not the lowest data qubits, a zoomed qubit, a three-block
+    chain whose middle tensor keeps edges beside its shared ones, the merge
+    pyramid and slices."""
+    c, probs = _chain(5, [14, 14], [4], most=1)
+    rng = np.random.default_rng(5)
+    roles = np.zeros(c.n_qubits, dtype=np.int8)
+    roles[rng.permutation(10)[:1]] = W.MERGED
+    roles[10 + rng.permutation(14)[:3]] = [W.ZOOM1, W.MERGED, W.MERGED]
+    _check(c, probs, roles)
+    c, probs = _chain(6, [8, 13, 8], [2, 2], most=1)
+    _check(c, probs, W.lowest_active_roles(c, [4, 11, 5]))
+    c, probs = _chain(7, [15, 14], [3], most=1)
+    for cfg in ({"merge_pyramid": True}, {"slice_edges": 1}):
+        _check(c, probs, W.lowest_active_roles(c, [12, 12]), **cfg)
+
+
+@pytest.mark.parametrize("widths,cuts,active,zoom", [
+    ([14, 13, 12], [1, 1], [1, 1, 0], {}),          # 2^11-state runs at the edge, 2^12 and 2^12
+    ([15, 14], [2], [2, 0], {0: 1, 13: 0}),
+    ([14], [], [1], {}),                             # one subcircuit: straight into the bins
+])
+def test_long_merge(widths, cuts, active, zoom):
+    c, probs = _chain(sum(widths), widths, cuts, ones=40)
+    for out in ("float32", "float64"):
+        _check(c, probs, W.lowest_active_roles(c, active, zoom), out=out)
