@@ -126,6 +126,9 @@ struct Plan {
 struct Batch {
   void* work = nullptr;
   size_t work_bytes = 0;
+  const BatchItem* merge_items = nullptr;   // the merges' launch
+  int64_t n_merge = 0;
+  bool merge_tiled = false;
   BatchLaunch L{};                   // phase 0 (the only phase of an FP32 batch)
   int grid = 0;
   std::vector<sqc_query_id> queries;
@@ -296,6 +299,10 @@ cudaError_t zero(sqc_ctx* ctx, void* dst, size_t bytes) {
 }
 
 inline int popc32(uint32_t x) { return __builtin_popcount(x); }
+
+// Whether a step may write C in 16-byte words (the plan's own tensors are
+// aligned; a caller's output need not be).
+bool aligned16(const void* C) { return (reinterpret_cast<uintptr_t>(C) & 15) == 0; }
 
 // Limit of every bounded device wait, from the configuration.
 uint64_t wait_ns(const sqc_ctx* ctx) {
@@ -1434,6 +1441,11 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
   struct TcPending { GemmTcArgs a; int phase; bool sums; int query; };
   std::vector<TcPending> tcs;
   int n_phases = 1;
+  // the merges run as a launch of their own ahead of the steps', except in a
+  // single query's one launch
+  const bool apart = !solo;
+  std::vector<char> merged;                  // per tensor slot: written by that launch
+  bool any_tiled = false;
   for (int j = 0; j < n; ++j) {
     Query& q = *qv[j];
     auto cit = ctx->circuits.find(q.circuit);
@@ -1457,14 +1469,21 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
       if (int(t) == P.final_tensor) continue;
       slot[t] = int(expected.size());
       expected.push_back(0);
+      merged.push_back(apart && P.tensors[t].producer_sub >= 0);
       slot_phase.push_back(0);
     }
     for (int i = 0; i < c.nC; ++i) {
       const int di = int(mdescs.size());
       mdescs.push_back(P.merge_host[i]);
-      const int64_t nblk = merge_blocks_of(P.merge_host[i]);
-      for (int64_t b = 0; b < nblk; ++b) items.push_back({{kItemMerge, di, b, -1, -1, slot[i]}, 0, 0});
-      expected[slot[i]] = unsigned(nblk);
+      // a work item: blocks that read about 64 KB together
+      const MergeDesc& md = P.merge_host[i];
+      const int64_t nblk = merge_blocks_of(md);
+      const int64_t reads = ((md.rows << md.a) << (md.m + 2)) / nblk;
+      const int64_t per = std::max<int64_t>(1, std::min<int64_t>(16, 65536 / std::max<int64_t>(reads, 1)));
+      for (int64_t b = 0; b < nblk; b += per)
+        items.push_back({{kItemMerge, di, b, int(std::min(per, nblk - b)), -1, -1, slot[i]}, 0, 0});
+      expected[slot[i]] = apart ? 0u : unsigned((nblk + per - 1) / per);
+      any_tiled = any_tiled || md.tiled;
     }
     const double alpha = std::ldexp(1.0, -c.K);
     for (size_t si = 0; si < P.steps.size(); ++si) {
@@ -1490,7 +1509,7 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
         a.chunk = (last && out_kind == OUT_F64 && c.K >= ctx->cfg.fp64_chunk_min_edges &&
                    st.Kd > ctx->cfg.chunk_terms) ? ctx->cfg.chunk_terms : 0;
         a.err = P.err;
-        a.contig16 = st.contig16;
+        a.contig16 = st.contig16 && aligned16(C);
         a.pairs = ctx->cfg.tc_pairs;
         a.wait_ns = wait_ns(ctx);
         if (solo && last) return fail(ctx, SQC_EINVAL, "batch: a single-query launch runs FP32 steps only");
@@ -1514,7 +1533,7 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
       a.K = st.Kd;
       a.rowmap = st.rowmap;
       a.colmap = st.colmap;
-      a.vec4 = st.vec4;
+      a.vec4 = st.vec4 && aligned16(C);
       a.C = C;
       a.kind = kind;
       a.plane_stride = pstride;
@@ -1526,6 +1545,12 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
       int64_t bm = 0, bn = 0;
       bs.cfg = batch_tile_cfg(a.M, a.N, a.K, a.chunk > 0, a.chunk, &bm, &bn, ctx->batch_policy);
       bs.ntiles = ((a.M + bm - 1) / bm) * ((a.N + bn - 1) / bn);
+      // steps that mostly write: bands (from half a band's outputs on)
+      if (a.M * a.N >= kBandOutputs / 2) {
+        // (a single-query launch names its output per run, aligned or not)
+        bs.band = last && solo ? 0 : band_rows(a, batch_cfg_group(bs.cfg), kBandOutputs);
+        if (bs.band > 0) bs.ntiles = (a.M / bs.band) * (a.N / band_cols(a.N));
+      }
       if (last && (totals || solo)) {
         part_off.push_back(n_parts);
         bs.total = solo ? nullptr : totals + j;
@@ -1541,7 +1566,7 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
       // tensor-core result or an earlier phase's tensor is complete already
       auto dep = [&](int t) { return (!by_tc[t] && av_simt[t] == ph) ? slot[t] : -1; };
       for (int64_t t = 0; t < bs.ntiles; ++t)
-        items.push_back({{kItemGemm, si_b, t, dep(st.x), dep(st.y), last ? -1 : slot[st.z]}, lvl, ph});
+        items.push_back({{kItemGemm, si_b, t, 0, dep(st.x), dep(st.y), last ? -1 : slot[st.z]}, lvl, ph});
       if (!last) {
         expected[slot[st.z]] = unsigned(bs.ntiles);
         slot_phase[slot[st.z]] = ph;
@@ -1554,6 +1579,20 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
   std::stable_sort(items.begin(), items.end(), [](const Pending& a, const Pending& b) {
     return a.phase != b.phase ? a.phase < b.phase : a.level < b.level;
   });
+  // Nothing waits for the merges' launch: a step's wait on a tensor it wrote
+  // goes, except on the batch's last tensor (complete at zero counts), whose
+  // target sqc_batch_inject_stall raises.
+  int64_t n_merge = 0;
+  for (Pending& p : items) {
+    if (p.it.type == kItemMerge) {
+      n_merge += apart;
+      if (apart) p.it.out = -1;
+      continue;
+    }
+    const int last_slot = int(expected.size()) - 1;
+    if (p.it.dep0 >= 0 && merged[p.it.dep0] && p.it.dep0 != last_slot) p.it.dep0 = -1;
+    if (p.it.dep1 >= 0 && merged[p.it.dep1] && p.it.dep1 != last_slot) p.it.dep1 = -1;
+  }
   std::vector<int64_t> ph_begin(n_phases + 1, 0);
   for (const Pending& p : items) ph_begin[p.phase + 1] += 1;
   for (int j = 0; j < n_phases; ++j) ph_begin[j + 1] += ph_begin[j];
@@ -1605,8 +1644,9 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
   B->tc.assign(n_phases, {});
   for (int j = 0; j < n_phases; ++j) {
     BatchLaunch& L = B->phases[j];
-    L.items = reinterpret_cast<const BatchItem*>(base + o_items) + ph_begin[j];
-    L.n_items = ph_begin[j + 1] - ph_begin[j];
+    const int64_t first = ph_begin[j] + (j == 0 ? n_merge : 0);       // (the merges sort first)
+    L.items = reinterpret_cast<const BatchItem*>(base + o_items) + first;
+    L.n_items = ph_begin[j + 1] - first;
     L.mdescs = reinterpret_cast<const MergeDesc*>(base + o_md);
     L.steps = reinterpret_cast<const BatchStep*>(base + o_st);
     L.counts = reinterpret_cast<unsigned*>(base + o_cnt);
@@ -1631,6 +1671,9 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
     B->n_tc += 1;
   }
   // the last phase's counters re-arm every slot (they all start at zero)
+  B->merge_items = reinterpret_cast<const BatchItem*>(base + o_items);
+  B->n_merge = n_merge;
+  B->merge_tiled = any_tiled;
   B->L = B->phases[0];
   B->grid = B->phase_grid[0];
   B->expected = std::move(expected);
@@ -2254,7 +2297,8 @@ sqc_status reconstruct_stages(sqc_ctx* ctx, sqc_query_id qid, sqc_precision prec
     }
   }
 
-  if (!fused && precision == SQC_PREC_FP32 && ctx->cfg.fused_query && P.n_slices == 1 && !P.steps.empty()) {
+  if (!fused && precision == SQC_PREC_FP32 && ctx->cfg.fused_query && P.n_slices == 1 && !P.steps.empty() &&
+      aligned16(out_bins)) {
     // the merge and every contraction step in ONE persistent launch: merge
     // blocks and step tiles form a dependency-ordered work list, each item
     // waiting only for the tensors it reads (the batched level's kernel
@@ -2336,7 +2380,7 @@ sqc_status reconstruct_stages(sqc_ctx* ctx, sqc_query_id qid, sqc_precision prec
         a.counter = P.counter;
         a.total = total_prob;
         a.err = P.err;
-        a.contig16 = st.contig16;
+        a.contig16 = st.contig16 && aligned16(C);
         a.pairs = ctx->cfg.tc_pairs;
         a.wait_ns = wait_ns(ctx);
         CK(launch_gemm_tc(a, s));
@@ -2349,7 +2393,7 @@ sqc_status reconstruct_stages(sqc_ctx* ctx, sqc_query_id qid, sqc_precision prec
         a.K = st.Kd;
         a.rowmap = st.rowmap;
         a.colmap = st.colmap;
-        a.vec4 = st.vec4;
+        a.vec4 = st.vec4 && aligned16(C);
         a.C = C;
         a.kind = kind;
         a.plane_stride = last ? 0 : Z.plane_stride;
@@ -2433,6 +2477,10 @@ SQC_API sqc_status sqc_batch_run(sqc_ctx* ctx, sqc_batch_id b, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StageScope scope(ctx, s, SQC_STAGE_CONTRACT);
   const Batch& B = *it->second;
+  if (B.n_merge > 0) {
+    CK(launch_batch_merges(B.merge_items, B.n_merge, B.L.mdescs, B.merge_tiled, s));
+    ctx->launches += 1;
+  }
   for (size_t j = 0; j < B.phases.size(); ++j) {
     if (B.phases[j].n_items > 0) {
       CK(launch_batch(B.phases[j], B.phase_grid[j], s));

@@ -112,8 +112,11 @@ __global__ void __launch_bounds__(kOpThreads, 2) batch_kernel(BatchLaunch L) {
     __syncthreads();
     if (!skip) {
       if (item.type == kItemMerge) {
-        if (md.tiled) merge_tile(md, item.tile, smem);
-        else merge_block(md, item.tile);
+        for (int b = 0; b < item.count; ++b) {
+          if (md.tiled) merge_tile(md, item.tile + b, smem);
+          else merge_block(md, item.tile + b);
+          if (md.tiled) __syncthreads();
+        }
       } else {
         const BatchStep& st = L.steps[item.idx];
         // a single-query launch names its output and probability sum per
@@ -121,7 +124,15 @@ __global__ void __launch_bounds__(kOpThreads, 2) batch_kernel(BatchLaunch L) {
         void* C = st.from_launch ? L.out : st.a.C;
         double* total = st.from_launch ? L.total : st.total;
         double mine;
-        switch (st.cfg) {
+        if (st.band > 0) {
+          const int64_t cols = st.a.N / band_cols(st.a.N);
+          const int c_shift = __ffsll(cols) - 1;
+          const int64_t m0 = (item.tile >> c_shift) * st.band, n0 = (item.tile & (cols - 1)) * band_cols(st.a.N);
+          // the FP32 groups of the probability check are the tile's
+          if (st.cfg == 2) mine = gemm_band<8, true>(st.a, m0, n0, st.band, smem, C);
+          else if (st.cfg == 1 || st.cfg == 4) mine = gemm_band<4, true>(st.a, m0, n0, st.band, smem, C);
+          else mine = gemm_band<2, true>(st.a, m0, n0, st.band, smem, C);
+        } else switch (st.cfg) {
           case 0: mine = run_tile<32, 32, 2, 2, false, 16>(st, item.tile, smem, C); break;
           case 1: mine = run_tile<64, 64, 4, 4, false, 16>(st, item.tile, smem, C); break;
           case 2: mine = run_tile<128, 64, 8, 4, false, 16>(st, item.tile, smem, C); break;
@@ -156,11 +167,48 @@ __global__ void __launch_bounds__(kOpThreads, 2) batch_kernel(BatchLaunch L) {
   }
 }
 
+// The merges of a level, one work item (some blocks of one descriptor) per
+// CTA.  On their own because they need a quarter of the steps' registers:
+// eight CTAs per SM cover the descriptor and item loads and the short chains
+// of each sum, where the steps' kernel holds two.  The states come from L2
+// (the resident tensors of a level's circuits fit it), so L2 bandwidth is the
+// bound.
+template <bool TILED>
+__global__ void __launch_bounds__(256) batch_merge_kernel(const BatchItem* __restrict__ items,
+                                                          const MergeDesc* __restrict__ mdescs) {
+  pdl_wait();      // the previous kernel on the stream has completed
+  pdl_trigger();   // the next one may start launching
+  __shared__ MergeDesc d;
+  __shared__ __align__(16) float tile[TILED ? kMergeTileFloats : 4];
+  const BatchItem it = items[blockIdx.x];
+  static_assert(sizeof(MergeDesc) % 8 == 0 && sizeof(MergeDesc) / 8 <= 256, "one word per thread");
+  if (threadIdx.x < sizeof(MergeDesc) / 8)
+    reinterpret_cast<uint64_t*>(&d)[threadIdx.x] = reinterpret_cast<const uint64_t*>(mdescs + it.idx)[threadIdx.x];
+  __syncthreads();
+  for (int b = 0; b < it.count; ++b) {
+    if (TILED && d.tiled) {
+      merge_tile(d, it.tile + b, tile);
+      __syncthreads();
+    } else {
+      merge_block(d, it.tile + b);
+    }
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_batch_merges(const BatchItem* items, int64_t n, const MergeDesc* mdescs, bool tiled,
+                                cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  return launch_k(tiled ? batch_merge_kernel<true> : batch_merge_kernel<false>, dim3(unsigned(n)), dim3(256), 0, s,
+                  false, items, mdescs);
+}
 
 int batch_smem_bytes() {
   // largest tile stage among the configurations above (64x64 with BK = 64)
-  return int(sizeof(float)) * gemm_tile_smem_floats<64, 64, 64>();
+  // and a band's rows
+  constexpr int f = gemm_tile_smem_floats<64, 64, 64>();
+  return int(sizeof(float)) * (f > kBandSmemFloats ? f : kBandSmemFloats);
 }
 
 cudaError_t batch_configure() {

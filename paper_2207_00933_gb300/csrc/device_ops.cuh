@@ -7,8 +7,6 @@
 
 namespace sqc {
 
-constexpr int kOpThreads = 256;
-
 // One lane's share of the sum over output (row of A, bin b) of descriptor d:
 // every lanes-th 16-byte word of the run (or every lanes-th value).
 __device__ __forceinline__ float merge_sum(const MergeDesc& d, const float* row, uint32_t b, uint32_t lane,
@@ -193,13 +191,15 @@ __device__ __forceinline__ void merge_block(const MergeDesc& d, int64_t blk) {
   const int64_t total = d.rows << d.a;
   const bool valid = o < total;
   float acc = 0.f;
-  if (valid) acc = merge_sum(d, merge_row(d, o >> d.a), uint32_t(o & ((int64_t(1) << d.a) - 1)), lane, lanes);
-  for (int off = lanes >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if (valid && lane == 0) {
+  uint64_t at = 0;
+  if (valid) {
     const int64_t e = o >> d.a;
     const uint32_t b = uint32_t(o & ((int64_t(1) << d.a) - 1));
-    store_out_f(d.dst, d.kind, d.plane_stride, d.rowmap[e] + d.colmap[b], acc * pow2_to_float(d.alpha));
+    at = __ldg(d.rowmap + e) + __ldg(d.colmap + b);   // on their way with the states
+    acc = merge_sum(d, merge_row(d, e), b, lane, lanes);
   }
+  for (int off = lanes >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+  if (valid && lane == 0) store_out_f(d.dst, d.kind, d.plane_stride, at, acc * pow2_to_float(d.alpha));
 }
 
 // Shared memory (floats) one SIMT tile needs for its A and B stages.
@@ -519,6 +519,107 @@ __device__ __forceinline__ double gemm_tile_pipe(const GemmArgs& a, int64_t m0, 
     sum += double(store_tile_f32<8, TN>(a, reinterpret_cast<const float(&)[8][TN]>(acc[i]), m0 + ty * TM + i,
                                         n0 + tx * TN, pow2_to_float(a.alpha), Cout));
   return sum;
+}
+
+
+// A band of a short shared index (K = 1, 4 or 16) with contiguous output
+// columns (vec4) and FP32 output: every thread keeps four columns' B rows in
+// registers and walks down the band's rows, whose A values it reads from
+// shared memory (each doubled, so that two columns' multiply-adds are one
+// instruction) -- 16 bytes stored per row, nothing else.  Such steps write
+// far more than they read or multiply; in 32 x 32 tiles each thread stores
+// four single floats after three dependent memory round trips.  k runs
+// upwards, with the zero term that a shared index below the plain tile's
+// stage of 16 gets there (it turns -0 into +0): the values are the same bit
+// for bit.  The probability check's FP32 groups are the plain tile's too: G
+// rows x 4 columns, or (G = 2) 2 x 2.
+//
+// Threads: CT = min(256, N / 4) across the columns, 256 / CT row groups; the
+// band is bm rows (a multiple of G * 256 / CT) x 4 CT columns.  smem: 2 bm K
+// floats and bm 8-byte offsets.
+template <int K, int G, bool CG>
+__device__ __forceinline__ double gemm_band_k(const GemmArgs& a, int64_t m0, int64_t n0, int bm, float* smem,
+                                              void* Cout) {
+  const int bn = band_cols(a.N), ct = bn >> 2, ct_log2 = __ffs(ct) - 1;
+  const int tid = threadIdx.x, col = 4 * (tid & (ct - 1)), rg = tid >> ct_log2, nrg = kOpThreads >> ct_log2;
+  float2* xs = reinterpret_cast<float2*>(smem);                       // [bm][K], doubled
+  uint64_t* roff = reinterpret_cast<uint64_t*>(smem + 2 * bm * K);    // [bm]
+  const uint64_t coff = __ldg(a.colmap + n0 + col);
+  float2 y[K][2];
+  {
+    const float* Y = a.B + (n0 + col) * K;
+    if constexpr (K >= 4) {
+#pragma unroll
+      for (int q = 0; q < K / 4; ++q) {
+        float4 w[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float4* p = reinterpret_cast<const float4*>(Y + c * K) + q;
+          if constexpr (CG) w[c] = __ldcg(p); else w[c] = __ldg(p);
+        }
+        y[4 * q][0] = make_float2(w[0].x, w[1].x); y[4 * q][1] = make_float2(w[2].x, w[3].x);
+        y[4 * q + 1][0] = make_float2(w[0].y, w[1].y); y[4 * q + 1][1] = make_float2(w[2].y, w[3].y);
+        y[4 * q + 2][0] = make_float2(w[0].z, w[1].z); y[4 * q + 2][1] = make_float2(w[2].z, w[3].z);
+        y[4 * q + 3][0] = make_float2(w[0].w, w[1].w); y[4 * q + 3][1] = make_float2(w[2].w, w[3].w);
+      }
+    } else {
+      y[0][0] = make_float2(ld_operand<CG>(Y), ld_operand<CG>(Y + 1));
+      y[0][1] = make_float2(ld_operand<CG>(Y + 2), ld_operand<CG>(Y + 3));
+    }
+  }
+  for (int i = tid; i < bm * K; i += kOpThreads) {
+    const float x = ld_operand<CG>(a.A + m0 * K + i);
+    xs[i] = make_float2(x, x);
+  }
+  for (int i = tid; i < bm; i += kOpThreads) roff[i] = __ldg(a.rowmap + m0 + i);
+  __syncthreads();
+  const float alpha = pow2_to_float(a.alpha);
+  float* out = static_cast<float*>(Cout) + coff;
+  float s_hi = 0.f, s_lo = 0.f;
+  for (int r0 = rg * G; r0 < bm; r0 += nrg * G) {
+    float g0 = 0.f, g1 = 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const float2* x = xs + (r0 + g) * K;
+      float2 c0 = make_float2(0.f, 0.f), c1 = make_float2(0.f, 0.f);
+      if constexpr (K >= 4) {
+#pragma unroll
+        for (int k = 0; k < K; k += 2) {
+          const float4 w = *reinterpret_cast<const float4*>(x + k);
+          fma2(c0, make_float2(w.x, w.y), y[k][0]);
+          fma2(c1, make_float2(w.x, w.y), y[k][1]);
+          fma2(c0, make_float2(w.z, w.w), y[k + 1][0]);
+          fma2(c1, make_float2(w.z, w.w), y[k + 1][1]);
+        }
+      } else {
+        fma2(c0, x[0], y[0][0]);
+        fma2(c1, x[0], y[0][1]);
+      }
+      if constexpr (K < 16) {
+        fma2(c0, make_float2(0.f, 0.f), make_float2(0.f, 0.f));
+        fma2(c1, make_float2(0.f, 0.f), make_float2(0.f, 0.f));
+      }
+      const float4 v = make_float4(c0.x * alpha, c0.y * alpha, c1.x * alpha, c1.y * alpha);
+      *reinterpret_cast<float4*>(out + roff[r0 + g]) = v;
+      if constexpr (G == 2) {
+        g0 = (g0 + v.x) + v.y;
+        g1 = (g1 + v.z) + v.w;
+      } else {
+        g0 += (v.x + v.y) + (v.z + v.w);
+      }
+    }
+    two_sum_add(s_hi, s_lo, g0);
+    if constexpr (G == 2) two_sum_add(s_hi, s_lo, g1);
+  }
+  __syncthreads();                                   // the next band may reuse the shared memory
+  return double(s_hi) + double(s_lo);
+}
+template <int G, bool CG>
+__device__ __forceinline__ double gemm_band(const GemmArgs& a, int64_t m0, int64_t n0, int bm, float* smem,
+                                            void* Cout) {
+  if (a.K == 16) return gemm_band_k<16, G, CG>(a, m0, n0, bm, smem, Cout);
+  if (a.K == 4) return gemm_band_k<4, G, CG>(a, m0, n0, bm, smem, Cout);
+  return gemm_band_k<1, G, CG>(a, m0, n0, bm, smem, Cout);
 }
 
 

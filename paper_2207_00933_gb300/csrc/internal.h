@@ -187,6 +187,25 @@ struct GemmArgs {
 cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t s);
 cudaError_t gemm_simt_configure();   // one-time kernel attributes (dynamic shared memory)
 
+constexpr int kOpThreads = 256;                  // threads of a contraction tile's or band's CTA
+// Bands of a step with a short shared index (gemm_band, device_ops.cuh).
+constexpr int kBandOutputs = 8192;               // outputs per band, as far as M allows
+constexpr int kBandSmemFloats = 2 * 4096 + 2 * 1024;
+__host__ __device__ inline int band_cols(int64_t N) { return N < 1024 ? int(N) : 1024; }
+// Rows of a band of a step (0: the step does not take bands): `outputs` per
+// band or fewer.
+inline int band_rows(const GemmArgs& a, int g, int64_t outputs) {
+  if (!a.vec4 || a.kind != OUT_F32 || a.chunk > 0 || a.accumulate || a.N < 16) return 0;
+  if (a.K != 1 && a.K != 4 && a.K != 16) return 0;
+  if ((reinterpret_cast<uintptr_t>(a.B) | reinterpret_cast<uintptr_t>(a.C)) & 15) return 0;
+  const int64_t bn = band_cols(a.N), least = int64_t(g) * (kOpThreads / (bn >> 2));
+  int64_t bm = outputs / bn;
+  if (bm > a.M) bm = a.M;
+  while (bm * a.K > 4096 || bm > 1024) bm >>= 1;
+  if (bm < least) bm = least;
+  return bm <= a.M && bm * a.K <= 4096 && bm <= 1024 ? int(bm) : 0;
+}
+
 // ---- contraction step, split-BF16 on tcgen05 ---------------------------------
 struct GemmTcArgs {
   const void* A;            // bf16 planes [3][Mp][Kp] (hi, mid, lo), K-contiguous
@@ -220,13 +239,15 @@ enum : int { kItemMerge = 0, kItemGemm = 1 };
 struct BatchItem {
   int type;          // kItemMerge / kItemGemm
   int idx;           // merge descriptor or step index in the batch arrays
-  int64_t tile;      // merge block (relative to the descriptor) or output tile
+  int64_t tile;      // first merge block (relative to the descriptor) or output tile
+  int count;         // merge blocks
   int dep0, dep1;    // tensor slots that must be complete first (-1: none)
   int out;           // tensor slot this item writes (-1: none)
 };
 struct BatchStep {
   GemmArgs a;        // a.partials != null: the query's last step (probability sum)
   int cfg;           // tile configuration id (batch_tile_cfg)
+  int band;          // > 0: bands of this many rows instead (gemm_band)
   int from_launch;   // the output and the probability sum are BatchLaunch::out / total
   int64_t ntiles;
   double* partials;  // per-tile partial sums of the query's bins
@@ -250,12 +271,18 @@ struct BatchLaunch {
   double* total;             // their probability sum (nullable)
 };
 cudaError_t launch_batch(const BatchLaunch& L, int grid, cudaStream_t s);
+// The merges of a batch as a launch of their own ahead of the steps': n items
+// (type merge, no dependencies), one per CTA; tiled: some descriptor is.
+cudaError_t launch_batch_merges(const BatchItem* items, int64_t n, const MergeDesc* mdescs, bool tiled,
+                                cudaStream_t s);
 cudaError_t batch_configure();
 int batch_smem_bytes();
 // tile configuration for a step of the batch kernel; *bm, *bn its tile
 int batch_tile_cfg(int64_t M, int64_t N, int64_t K, bool chunked, int64_t chunk, int64_t* bm, int64_t* bn,
                    int policy);
 constexpr int kBatchPolicies = 3;
+// rows of the FP32 groups of a configuration's probability sum (gemm_band)
+inline int batch_cfg_group(int cfg) { return cfg == 2 ? 8 : (cfg == 1 || cfg == 4 ? 4 : 2); }
 
 // ---- probability check: FP64 sum of n values ---------------------------------
 cudaError_t launch_sum(const void* x, int is_f64, uint64_t n, double* partials, unsigned* counter,

@@ -218,10 +218,13 @@ bool sqc_server::dispatch(Slot& sl, int idx) {
       st = sqc_reconstruct(ctx, qs[j], SQC_PREC_FP32, outs[j], SQC_F32, size_t(4) << nas[j], nullptr, sl.s);
   } else {
     // the batch's own state is allocated last: if it does not fit, hand the
-    // most recently admitted requests back to the queue and retry
+    // most recently admitted requests back to the queue and retry -- the only
+    // one too while other launches hold memory
+    bool others = false;
+    for (const Slot& o : slots) others = others || o.busy;
     for (;;) {
       st = sqc_batch_create(ctx, int32_t(qs.size()), qs.data(), outs.data(), SQC_F32, nullptr, SQC_PREC_FP32, &sl.b);
-      if (st != SQC_EBUSY || qs.size() == 1) break;
+      if (st != SQC_EBUSY || (qs.size() == 1 && !others)) break;
       ++busy_refusals;
       sqc::ctx_free(ctx, outs.back(), size_t(4) << nas.back());
       sqc_release_query(ctx, qs.back());
@@ -237,6 +240,7 @@ bool sqc_server::dispatch(Slot& sl, int idx) {
       qs.pop_back();
       outs.pop_back();
       nas.pop_back();
+      if (qs.empty()) return false;            // waits for launches to retire
     }
     if (st == SQC_OK) {
       sl.has_batch = true;

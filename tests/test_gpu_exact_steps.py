@@ -106,3 +106,43 @@ def test_long_merge(widths, cuts, active, zoom):
     c, probs = _chain(sum(widths), widths, cuts, ones=40)
     for out in ("float32", "float64"):
         _check(c, probs, W.lowest_active_roles(c, active, zoom), out=out)
+
+
+@pytest.mark.parametrize("policy", [0, 2])
+def test_batch_bands(policy):
+    """The batched launch's bands (shared index 1, 4 and 16, from the smallest
+    to several bands, more rows than columns and fewer) and its merges, for
+    queries of one launch that differ in every shape; and an output that is
+    not 16-byte aligned, which takes the plain tiles."""
+    import torch
+    from paper_2207_00933_gb300 import Context, _build
+    _build.build()
+    shapes = [([7, 7], [1], [6, 7]), ([7, 8], [2], [5, 8]), ([9, 12], [1], [5, 11]), ([12, 9], [2], [10, 4]),
+              ([5, 14], [2], [3, 12]), ([13, 5], [1], [12, 3]), ([8, 9, 8], [1, 2], [5, 5, 6]), ([9, 9], [0], [6, 8]),
+              ([10, 10, 9], [2, 2], [4, 3, 5]), ([12, 12], [2], [9, 9]), ([13, 13], [2], [11, 11])]
+    with Context(0) as ctx:
+        queries, outs, want, store = [], [], [], []
+        for j, (widths, cuts, active) in enumerate(shapes):
+            c, probs = _chain(100 + j, widths, cuts, most=1)
+            roles = W.lowest_active_roles(c, active)
+            cid = ctx.load_subcircuit_outputs(c.n_qubits, *c.graph_arrays(), [torch.from_numpy(p).cuda() for p in probs])
+            q, na = ctx.set_qubit_roles(cid, roles)
+            buf = torch.full(((1 << na) + 1,), float("nan"), dtype=torch.float32, device="cuda")
+            queries.append(q)
+            store.append(buf)
+            outs.append(buf[j == 3:][:1 << na])
+            g = O.Graph.from_arrays(c.n_qubits, *c.graph_arrays())
+            T = O.subcircuit_tensors(g, [p.astype(np.float64) for p in probs], roles)
+            assert O.reconstruct_pairwise(g, [np.abs(t) for t in T], roles).max() * 2.0 ** c.n_edges < 2 ** 24
+            want.append(O.reconstruct_pairwise(g, T, roles))
+        totals = torch.zeros(len(queries), dtype=torch.float64, device="cuda")
+        if policy:
+            ctx.batch_autotune(queries, outs, totals, reps=1)
+        b = ctx.batch_create(queries, outs, totals)
+        for _ in range(2):
+            ctx.batch_run(b)
+        ctx.batch_status(b)
+        for o, w, t in zip(outs, want, totals.cpu().numpy()):
+            assert np.array_equal(o.double().cpu().numpy(), w)
+            assert abs(t - w.sum()) <= 1e-6 * np.abs(w).sum()
+        ctx.batch_release(b)
