@@ -1479,7 +1479,8 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
       const MergeDesc& md = P.merge_host[i];
       const int64_t nblk = merge_blocks_of(md);
       const int64_t reads = ((md.rows << md.a) << (md.m + 2)) / nblk;
-      const int64_t per = std::max<int64_t>(1, std::min<int64_t>(16, 65536 / std::max<int64_t>(reads, 1)));
+      const int64_t most = reads < 8192 ? 4 : 16;      // (small blocks: enough CTAs to overlap their latency)
+      const int64_t per = std::max<int64_t>(1, std::min<int64_t>(most, 65536 / std::max<int64_t>(reads, 1)));
       for (int64_t b = 0; b < nblk; b += per)
         items.push_back({{kItemMerge, di, b, int(std::min(per, nblk - b)), -1, -1, slot[i]}, 0, 0});
       expected[slot[i]] = apart ? 0u : unsigned((nblk + per - 1) / per);
@@ -1549,7 +1550,7 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
       if (a.M * a.N >= kBandOutputs / 2) {
         // (a single-query launch names its output per run, aligned or not)
         bs.band = last && solo ? 0 : band_rows(a, batch_cfg_group(bs.cfg), kBandOutputs);
-        if (bs.band > 0) bs.ntiles = (a.M / bs.band) * (a.N / band_cols(a.N));
+        if (bs.band > 0) bs.ntiles = (a.M / bs.band) * (a.N / band_cols(a));
       }
       if (last && (totals || solo)) {
         part_off.push_back(n_parts);

@@ -33,25 +33,27 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
 }
 
 // Per-query FP64 probability sum over the final step's tiles: each tile
-// stores its partial, the last one adds them in tile order into *total.
-__device__ __forceinline__ void finish_query_total(double mine, const BatchStep& st, int64_t tile, double* total,
-                                                   double* red) {
-  __shared__ bool is_last;
-  const double bs = block_sum(mine, red);
-  if (threadIdx.x == 0) {
-    st.partials[tile] = bs;
+// stores its partial (the warps' sums in red, added in warp order), the last
+// one adds them into *total in a fixed order.  Run by one warp while the rest
+// of the CTA goes on to the next item.
+__device__ __forceinline__ void finish_query_total(const double* red, const BatchStep& st, int64_t tile,
+                                                   double* total) {
+  const int lane = threadIdx.x & 31;
+  int last = 0;
+  if (lane == 0) {
+    double s = 0.0;
+    for (int w = 0; w < kOpThreads / 32; ++w) s += red[w];
+    st.partials[tile] = s;
     __threadfence();
-    const unsigned t = atomicAdd(st.counter, 1u);
-    is_last = (t == unsigned(st.ntiles - 1));
+    last = atomicAdd(st.counter, 1u) == unsigned(st.ntiles - 1);
   }
-  __syncthreads();
-  if (!is_last) return;
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
   __threadfence();
   double s = 0.0;
-  for (int64_t i = threadIdx.x; i < st.ntiles; i += blockDim.x) s += static_cast<volatile double*>(st.partials)[i];
-  const double tot = block_sum(s, red);
-  if (threadIdx.x == 0) {
-    *total = tot;
+  for (int64_t i = lane; i < st.ntiles; i += 32) s += static_cast<volatile double*>(st.partials)[i];
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (lane == 0) {
+    *total = s;
     *st.counter = 0u;
   }
 }
@@ -72,45 +74,76 @@ __global__ void __launch_bounds__(kOpThreads, 2) batch_kernel(BatchLaunch L) {
   pdl_trigger();   // the next one may start launching
   extern __shared__ __align__(16) float smem[];
   __shared__ MergeDesc md;
-  __shared__ BatchItem item;
-  __shared__ int64_t my;
+  __shared__ __align__(16) BatchItem items[2];
   __shared__ double red[kOpThreads / 32];
   __shared__ bool is_last;
-  __shared__ int skip;
-  for (;;) {
+  __shared__ int skip;                        // -1: no more items
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // Items are claimed one ahead, so that an item's number and contents are on
+  // their way while the one before it is worked on.  Every CTA works through
+  // its claims in list order, so the earliest unfinished item is never held
+  // up by a later one and the schedule still cannot deadlock.
+  auto claim = [&]() -> int64_t {
+    return int64_t(atomicAdd(reinterpret_cast<unsigned long long*>(L.head), 1ull));
+  };
+  int64_t id = 0, next = 0;                   // thread 0: this item's number and the next one's
+  if (threadIdx.x == 0) {
+    id = claim();
+    next = claim();
+    if (id < L.n_items) items[0] = L.items[id];
+  }
+  for (int p = 0;; p ^= 1) {
+    const BatchItem& item = items[p];
     if (threadIdx.x == 0) {
-      my = (*static_cast<volatile int*>(L.abort)) ? L.n_items : int64_t(atomicAdd(reinterpret_cast<unsigned long long*>(L.head), 1ull));
-      if (my < L.n_items) item = L.items[my];
-    }
-    __syncthreads();
-    if (my >= L.n_items) break;
-    if (threadIdx.x == 0) {
-      // wait for the input tensors (bounded; abort on timeout)
-      for (int k = 0; k < 2; ++k) {
-        const int dep = k ? item.dep1 : item.dep0;
-        if (dep < 0) continue;
-        uint32_t i = 0;
-        uint64_t t0 = 0;
-        while (ld_acquire(L.counts + dep) < L.expected[dep]) {
-          if (*static_cast<volatile int*>(L.abort)) break;     // another CTA gave up: drain
-          if ((++i & 31) == 0) {
-            const uint64_t now = global_ns();
-            if (t0 == 0) {
-              t0 = now;
-            } else if (now - t0 > L.wait_ns) {
-              atomicExch(L.abort, 1);
-              atomicExch(L.err, 1);
-              break;
-            }
-          }
-          if (i > 32) __nanosleep(64);
+      skip = -1;
+      if (id < L.n_items) {
+        // wait for the input tensors (bounded; abort on timeout)
+        unsigned want[2], have[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int dep = k ? item.dep1 : item.dep0;
+          want[k] = dep < 0 ? 0u : __ldg(L.expected + dep);
+          have[k] = dep < 0 ? 0u : ld_acquire(L.counts + dep);
         }
+        for (int k = 0; k < 2; ++k) {
+          const int dep = k ? item.dep1 : item.dep0;
+          uint32_t i = 0;
+          uint64_t t0 = 0;
+          while (have[k] < want[k]) {
+            if (*static_cast<volatile int*>(L.abort)) break;     // another CTA gave up: drain
+            if ((++i & 31) == 0) {
+              const uint64_t now = global_ns();
+              if (t0 == 0) {
+                t0 = now;
+              } else if (now - t0 > L.wait_ns) {
+                atomicExch(L.abort, 1);
+                atomicExch(L.err, 1);
+                break;
+              }
+            }
+            if (i > 32) __nanosleep(64);
+            have[k] = ld_acquire(L.counts + dep);
+          }
+        }
+        if (item.type == kItemMerge) md = L.mdescs[item.idx];
+        skip = *static_cast<volatile int*>(L.abort) ? 1 : 0;    // one decision for the whole CTA
       }
-      if (item.type == kItemMerge) md = L.mdescs[item.idx];
-      skip = *static_cast<volatile int*>(L.abort);    // one decision for the whole CTA
     }
     __syncthreads();
-    if (!skip) {
+    const int sk = skip;
+    if (sk < 0) break;
+    if (threadIdx.x == 0) {
+      if (next < L.n_items) {
+        const char* src = reinterpret_cast<const char*>(L.items + next);
+        const uint32_t dst = uint32_t(__cvta_generic_to_shared(&items[p ^ 1]));
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst + 16), "l"(src + 16) : "memory");
+      }
+      id = sk ? L.n_items : next;             // after an abort: drain
+      next = claim();
+    }
+    const BatchStep* sums = nullptr;          // a last step with a probability sum
+    if (!sk) {
       if (item.type == kItemMerge) {
         for (int b = 0; b < item.count; ++b) {
           if (md.tiled) merge_tile(md, item.tile + b, smem);
@@ -125,9 +158,9 @@ __global__ void __launch_bounds__(kOpThreads, 2) batch_kernel(BatchLaunch L) {
         double* total = st.from_launch ? L.total : st.total;
         double mine;
         if (st.band > 0) {
-          const int64_t cols = st.a.N / band_cols(st.a.N);
+          const int64_t cols = st.a.N / band_cols(st.a);
           const int c_shift = __ffsll(cols) - 1;
-          const int64_t m0 = (item.tile >> c_shift) * st.band, n0 = (item.tile & (cols - 1)) * band_cols(st.a.N);
+          const int64_t m0 = (item.tile >> c_shift) * st.band, n0 = (item.tile & (cols - 1)) * band_cols(st.a);
           // the FP32 groups of the probability check are the tile's
           if (st.cfg == 2) mine = gemm_band<8, true>(st.a, m0, n0, st.band, smem, C);
           else if (st.cfg == 1 || st.cfg == 4) mine = gemm_band<4, true>(st.a, m0, n0, st.band, smem, C);
@@ -141,14 +174,22 @@ __global__ void __launch_bounds__(kOpThreads, 2) batch_kernel(BatchLaunch L) {
           case 5: mine = run_tile<32, 32, 2, 2, true, 16>(st, item.tile, smem, C); break;
           default: mine = run_tile<64, 64, 4, 4, true, 16>(st, item.tile, smem, C); break;
         }
-        if (st.a.partials && total) finish_query_total(mine, st, item.tile, total, red);
+        if (st.a.partials && total) {
+          for (int off = 16; off > 0; off >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, off);
+          if (lane == 0) red[warp] = mine;
+          sums = &st;
+        }
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0 && item.out >= 0) {
-      __threadfence();
-      atomicAdd(L.counts + item.out, 1u);
+    if (warp == 1) {
+      if (sums) finish_query_total(red, *sums, item.tile, sums->from_launch ? L.total : sums->total);
+      if (lane == 0 && item.out >= 0) {
+        __threadfence();
+        atomicAdd(L.counts + item.out, 1u);
+      }
     }
+    if (threadIdx.x == 0) asm volatile("cp.async.wait_all;" ::: "memory");
   }
   // the last CTA out re-arms the schedule for the next launch
   if (threadIdx.x == 0) {
@@ -181,6 +222,7 @@ __global__ void __launch_bounds__(256) batch_merge_kernel(const BatchItem* __res
   __shared__ MergeDesc d;
   __shared__ __align__(16) float tile[TILED ? kMergeTileFloats : 4];
   const BatchItem it = items[blockIdx.x];
+  static_assert(sizeof(BatchItem) == 32, "fetched as two 16-byte words");
   static_assert(sizeof(MergeDesc) % 8 == 0 && sizeof(MergeDesc) / 8 <= 256, "one word per thread");
   if (threadIdx.x < sizeof(MergeDesc) / 8)
     reinterpret_cast<uint64_t*>(&d)[threadIdx.x] = reinterpret_cast<const uint64_t*>(mdescs + it.idx)[threadIdx.x];

@@ -191,15 +191,13 @@ __device__ __forceinline__ void merge_block(const MergeDesc& d, int64_t blk) {
   const int64_t total = d.rows << d.a;
   const bool valid = o < total;
   float acc = 0.f;
-  uint64_t at = 0;
-  if (valid) {
+  if (valid) acc = merge_sum(d, merge_row(d, o >> d.a), uint32_t(o & ((int64_t(1) << d.a) - 1)), lane, lanes);
+  for (int off = lanes >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+  if (valid && lane == 0) {
     const int64_t e = o >> d.a;
     const uint32_t b = uint32_t(o & ((int64_t(1) << d.a) - 1));
-    at = __ldg(d.rowmap + e) + __ldg(d.colmap + b);   // on their way with the states
-    acc = merge_sum(d, merge_row(d, e), b, lane, lanes);
+    store_out_f(d.dst, d.kind, d.plane_stride, d.rowmap[e] + d.colmap[b], acc * pow2_to_float(d.alpha));
   }
-  for (int off = lanes >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if (valid && lane == 0) store_out_f(d.dst, d.kind, d.plane_stride, at, acc * pow2_to_float(d.alpha));
 }
 
 // Shared memory (floats) one SIMT tile needs for its A and B stages.
@@ -290,46 +288,54 @@ __device__ __forceinline__ double gemm_tile(const GemmArgs& a, int64_t m0, int64
       for (int j = 0; j < TN; ++j) acc64[i][j] = 0.0;
   }
 
-  // the operand loads of a stage are issued in groups of four before their
-  // shared-memory stores, so that four are in flight together (one memory
-  // round trip per group instead of one per load; four keeps the registers
-  // of the deep tile shapes in bounds)
-  constexpr int kLA = (BM * kBK + kThreads - 1) / kThreads;
-  constexpr int kLB = (BN * kBK + kThreads - 1) / kThreads;
-  constexpr int kG = 4;
+  // A stage's operands: 16-byte words along the shared index, both operands'
+  // loads in flight before their shared-memory stores (one memory round trip
+  // per stage; four-byte loads in groups of four took up to eight).  A shared
+  // index of 1 (an outer product) has no such words.
+  constexpr int kQ = kBK / 4;
+  constexpr int kLA = (BM * kQ + kThreads - 1) / kThreads;
+  constexpr int kLB = (BN * kQ + kThreads - 1) / kThreads;
+  auto ld4 = [](const float* p) -> float4 {
+    if constexpr (CG) return __ldcg(reinterpret_cast<const float4*>(p));
+    else return __ldg(reinterpret_cast<const float4*>(p));
+  };
   for (int64_t k0 = 0; k0 < a.K; k0 += kBK) {
+    if (a.K >= 4) {
+      float4 ra[kLA], rb[kLB];
 #pragma unroll
-    for (int g0 = 0; g0 < kLA; g0 += kG) {
-      float rv[kG];
-#pragma unroll
-      for (int u = 0; u < kG; ++u) {
-        const int idx = tid + (g0 + u) * kThreads;
-        const int r = idx / kBK, kk = idx % kBK;
-        rv[u] = 0.f;
-        if (g0 + u < kLA && idx < BM * kBK && m0 + r < a.M && k0 + kk < a.K)
-          rv[u] = ld_operand<CG>(a.A + (m0 + r) * a.K + k0 + kk);
+      for (int u = 0; u < kLA; ++u) {
+        const int i = tid + u * kThreads, r = i / kQ, kk = 4 * (i % kQ);
+        ra[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < BM * kQ && m0 + r < a.M && k0 + kk < a.K) ra[u] = ld4(a.A + (m0 + r) * a.K + k0 + kk);
       }
 #pragma unroll
-      for (int u = 0; u < kG; ++u) {
-        const int idx = tid + (g0 + u) * kThreads;
-        if (g0 + u < kLA && idx < BM * kBK) As[idx % kBK][idx / kBK] = rv[u];
-      }
-    }
-#pragma unroll
-    for (int g0 = 0; g0 < kLB; g0 += kG) {
-      float rv[kG];
-#pragma unroll
-      for (int u = 0; u < kG; ++u) {
-        const int idx = tid + (g0 + u) * kThreads;
-        const int r = idx / kBK, kk = idx % kBK;
-        rv[u] = 0.f;
-        if (g0 + u < kLB && idx < BN * kBK && n0 + r < a.N && k0 + kk < a.K)
-          rv[u] = ld_operand<CG>(a.B + (n0 + r) * a.K + k0 + kk);
+      for (int u = 0; u < kLB; ++u) {
+        const int i = tid + u * kThreads, r = i / kQ, kk = 4 * (i % kQ);
+        rb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < BN * kQ && n0 + r < a.N && k0 + kk < a.K) rb[u] = ld4(a.B + (n0 + r) * a.K + k0 + kk);
       }
 #pragma unroll
-      for (int u = 0; u < kG; ++u) {
-        const int idx = tid + (g0 + u) * kThreads;
-        if (g0 + u < kLB && idx < BN * kBK) Bs[idx % kBK][idx / kBK] = rv[u];
+      for (int u = 0; u < kLA; ++u) {
+        const int i = tid + u * kThreads, r = i / kQ, kk = 4 * (i % kQ);
+        if (i < BM * kQ) {
+          As[kk][r] = ra[u].x; As[kk + 1][r] = ra[u].y; As[kk + 2][r] = ra[u].z; As[kk + 3][r] = ra[u].w;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kLB; ++u) {
+        const int i = tid + u * kThreads, r = i / kQ, kk = 4 * (i % kQ);
+        if (i < BN * kQ) {
+          Bs[kk][r] = rb[u].x; Bs[kk + 1][r] = rb[u].y; Bs[kk + 2][r] = rb[u].z; Bs[kk + 3][r] = rb[u].w;
+        }
+      }
+    } else {
+      for (int i = tid; i < BM * kBK; i += kThreads) {
+        const int r = i % BM, kk = i / BM;
+        As[kk][r] = kk == 0 && m0 + r < a.M ? ld_operand<CG>(a.A + m0 + r) : 0.f;
+      }
+      for (int i = tid; i < BN * kBK; i += kThreads) {
+        const int r = i % BN, kk = i / BN;
+        Bs[kk][r] = kk == 0 && n0 + r < a.N ? ld_operand<CG>(a.B + n0 + r) : 0.f;
       }
     }
     __syncthreads();
@@ -522,25 +528,23 @@ __device__ __forceinline__ double gemm_tile_pipe(const GemmArgs& a, int64_t m0, 
 }
 
 
-// A band of a short shared index (K = 1, 4 or 16) with contiguous output
-// columns (vec4) and FP32 output: every thread keeps four columns' B rows in
-// registers and walks down the band's rows, whose A values it reads from
-// shared memory (each doubled, so that two columns' multiply-adds are one
-// instruction) -- 16 bytes stored per row, nothing else.  Such steps write
-// far more than they read or multiply; in 32 x 32 tiles each thread stores
-// four single floats after three dependent memory round trips.  k runs
-// upwards, with the zero term that a shared index below the plain tile's
-// stage of 16 gets there (it turns -0 into +0): the values are the same bit
-// for bit.  The probability check's FP32 groups are the plain tile's too: G
-// rows x 4 columns, or (G = 2) 2 x 2.
+// Bands: steps of a short shared index (K = 1, 4 or 16) with contiguous output
+// columns (vec4) and FP32 output write far more than they read or multiply.
+// In plain tiles a thread stores a few values after a chain of dependent
+// memory round trips; a band's thread owns four columns and walks down the
+// band's rows, 16 bytes stored per row.  k runs upwards, with the zero term
+// that a shared index below the plain tile's stage of 16 gets there (it turns
+// -0 into +0): the values are the same bit for bit.  The probability check's
+// FP32 groups are the plain tile's too: G rows x 4 columns, or (G = 2) 2 x 2.
 //
-// Threads: CT = min(256, N / 4) across the columns, 256 / CT row groups; the
-// band is bm rows (a multiple of G * 256 / CT) x 4 CT columns.  smem: 2 bm K
-// floats and bm 8-byte offsets.
+// Threads: CT = columns / 4 across the columns, 256 / CT row groups.
+// K <= 4: a thread's four B rows stay in registers; A's rows are read from
+// shared memory, each value doubled, so that two columns' multiply-adds are
+// one instruction.  smem: 2 bm K floats and bm 8-byte offsets.
 template <int K, int G, bool CG>
 __device__ __forceinline__ double gemm_band_k(const GemmArgs& a, int64_t m0, int64_t n0, int bm, float* smem,
                                               void* Cout) {
-  const int bn = band_cols(a.N), ct = bn >> 2, ct_log2 = __ffs(ct) - 1;
+  const int bn = band_cols(a), ct = bn >> 2, ct_log2 = __ffs(ct) - 1;
   const int tid = threadIdx.x, col = 4 * (tid & (ct - 1)), rg = tid >> ct_log2, nrg = kOpThreads >> ct_log2;
   float2* xs = reinterpret_cast<float2*>(smem);                       // [bm][K], doubled
   uint64_t* roff = reinterpret_cast<uint64_t*>(smem + 2 * bm * K);    // [bm]
@@ -614,13 +618,99 @@ __device__ __forceinline__ double gemm_band_k(const GemmArgs& a, int64_t m0, int
   __syncthreads();                                   // the next band may reuse the shared memory
   return double(s_hi) + double(s_lo);
 }
+// K = 16: both operands in shared memory, k-major; 8 rows x 4 columns per
+// thread and round, the multiply-adds of two rows in one instruction (four B
+// rows of 16 in registers were loaded a line per lane, and took longer than
+// the stores).  smem: 16 (bm + 4) + 16 (bn + 4) floats and bm offsets.
+template <int G, bool CG>
+__device__ __forceinline__ double gemm_band_16(const GemmArgs& a, int64_t m0, int64_t n0, int bm, float* smem,
+                                               void* Cout) {
+  const int bn = band_cols(a), ct = bn >> 2, ct_log2 = __ffs(ct) - 1;
+  const int tid = threadIdx.x, col = 4 * (tid & (ct - 1)), rg = tid >> ct_log2, nrg = kOpThreads >> ct_log2;
+  const int sx = bm + 4, sy = bn + 4;
+  float* xs = smem;                                                   // [16][sx]
+  float* ys = smem + 16 * sx;                                         // [16][sy]
+  uint64_t* roff = reinterpret_cast<uint64_t*>(ys + 16 * sy);         // [bm]
+  const uint64_t coff = __ldg(a.colmap + n0 + col);
+  auto ld4 = [](const float* p) -> float4 {
+    if constexpr (CG) return __ldcg(reinterpret_cast<const float4*>(p));
+    else return __ldg(reinterpret_cast<const float4*>(p));
+  };
+  const float* X = a.A + m0 * 16;
+  const float* Y = a.B + n0 * 16;
+  // four 16-byte words in flight per thread (each row is four of them)
+  auto stage = [&](const float* src, int rows, float* dst, int stride) {
+    for (int i0 = tid; i0 < rows * 4; i0 += 4 * kOpThreads) {
+      float4 w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u * kOpThreads < rows * 4) w[u] = ld4(src + 4 * (i0 + u * kOpThreads));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * kOpThreads;
+        if (i < rows * 4) {
+          float* p = dst + 4 * (i & 3) * stride + (i >> 2);
+          p[0] = w[u].x; p[stride] = w[u].y; p[2 * stride] = w[u].z; p[3 * stride] = w[u].w;
+        }
+      }
+    }
+  };
+  stage(X, bm, xs, sx);
+  stage(Y, bn, ys, sy);
+  for (int i = tid; i < bm; i += kOpThreads) roff[i] = __ldg(a.rowmap + m0 + i);
+  __syncthreads();
+  const float alpha = pow2_to_float(a.alpha);
+  float* out = static_cast<float*>(Cout) + coff;
+  float s_hi = 0.f, s_lo = 0.f;
+  for (int r0 = rg * 8; r0 < bm; r0 += nrg * 8) {
+    float2 acc[4][4];                                // [row pair][column]
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[i][c] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int k = 0; k < 16; ++k) {
+      const float4 y = *reinterpret_cast<const float4*>(ys + k * sy + col);
+      const float4 x0 = *reinterpret_cast<const float4*>(xs + k * sx + r0);
+      const float4 x1 = *reinterpret_cast<const float4*>(xs + k * sx + r0 + 4);
+      const float2 xp[4] = {make_float2(x0.x, x0.y), make_float2(x0.z, x0.w), make_float2(x1.x, x1.y),
+                            make_float2(x1.z, x1.w)};
+      const float yc[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) fma2(acc[i][c], xp[i], make_float2(yc[c], yc[c]));
+    }
+    float g0 = 0.f, g1 = 0.f;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      float v[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] = (r & 1 ? acc[r >> 1][c].y : acc[r >> 1][c].x) * alpha;
+      *reinterpret_cast<float4*>(out + roff[r0 + r]) = make_float4(v[0], v[1], v[2], v[3]);
+      if constexpr (G == 2) {
+        g0 = (g0 + v[0]) + v[1];
+        g1 = (g1 + v[2]) + v[3];
+      } else {
+        g0 += (v[0] + v[1]) + (v[2] + v[3]);
+      }
+      if ((r + 1) % G == 0) {
+        two_sum_add(s_hi, s_lo, g0);
+        if constexpr (G == 2) two_sum_add(s_hi, s_lo, g1);
+        g0 = g1 = 0.f;
+      }
+    }
+  }
+  __syncthreads();                                   // the next band may reuse the shared memory
+  return double(s_hi) + double(s_lo);
+}
+
 template <int G, bool CG>
 __device__ __forceinline__ double gemm_band(const GemmArgs& a, int64_t m0, int64_t n0, int bm, float* smem,
                                             void* Cout) {
-  if (a.K == 16) return gemm_band_k<16, G, CG>(a, m0, n0, bm, smem, Cout);
+  if (a.K == 16) return gemm_band_16<G, CG>(a, m0, n0, bm, smem, Cout);
   if (a.K == 4) return gemm_band_k<4, G, CG>(a, m0, n0, bm, smem, Cout);
   return gemm_band_k<1, G, CG>(a, m0, n0, bm, smem, Cout);
 }
-
 
 }  // namespace sqc

@@ -51,6 +51,27 @@ __global__ void __launch_bounds__(kPipeThreads, 3) gemm_pipe_kernel(GemmArgs a) 
   if (a.partials) finish_total(mysum, a.partials, a.counter, a.total, red);
 }
 
+// Bands of a short shared index (gemm_band), one per CTA.
+template <int G>
+__global__ void __launch_bounds__(kThreads, 2) gemm_band_kernel(GemmArgs a, int bm) {
+  pdl_wait();      // the previous kernel on the stream has completed
+  pdl_trigger();   // the next one may start launching
+  __shared__ __align__(16) float smem[kBandSmemFloats];
+  __shared__ double red[kThreads / 32];
+  const int bn = band_cols(a);
+  const int c_shift = __ffsll(a.N / bn) - 1;
+  const int64_t tile = blockIdx.x;
+  const int64_t m0 = (tile >> c_shift) * bm, n0 = (tile & ((int64_t(1) << c_shift) - 1)) * bn;
+  const double mysum = gemm_band<G, false>(a, m0, n0, bm, smem, a.C);
+  if (a.partials) finish_total(mysum, a.partials, a.counter, a.total, red);
+}
+
+template <int G>
+cudaError_t launch_band(const GemmArgs& a, int bm, cudaStream_t s) {
+  return launch_k(gemm_band_kernel<G>, dim3(unsigned((a.M / bm) * (a.N / band_cols(a)))), dim3(kThreads), 0, s,
+                  false, a, bm);
+}
+
 template <int BM, int BN, int TM, int TN>
 cudaError_t launch_pipe(const GemmArgs& a, cudaStream_t s) {
   return launch_k(gemm_pipe_kernel<BM, BN, TM, TN>, dim3(unsigned((a.M / BM) * (a.N / BN))), dim3(kPipeThreads),
@@ -76,6 +97,10 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s) {
 
 }  // namespace
 
+namespace {
+constexpr int64_t kBandLeast = int64_t(1) << 18;
+}
+
 cudaError_t gemm_simt_configure() {
   return cudaFuncSetAttribute(gemm_pipe_kernel<128, 64, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               int(sizeof(float)) * gemm_pipe_smem_floats<128, 64>());
@@ -87,6 +112,18 @@ cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t s) {
   const bool wide = !chunked && a.kind == OUT_F32;
   auto tiles = [&](int bm, int bn) { return ((a.M + bm - 1) / bm) * ((a.N + bn - 1) / bn); };
   const int64_t want = 152;   // at least one full wave of CTAs
+  // bands (shared index up to 16, contiguous columns) once two per SM have
+  // 1024 outputs each; the FP32 groups of the probability check stay those of
+  // the plain tile the step would take
+  const int64_t outs = a.M * a.N;
+  if (wide && outs >= kBandLeast) {
+    int64_t per = kBandOutputs;
+    while (per > 1024 && outs / per < 2 * want) per >>= 1;
+    const int g = tiles(128, 128) >= want ? 8 : (tiles(64, 64) >= want ? 4 : 2);
+    const int bm = band_rows(a, g, per);
+    if (bm > 0 && (a.M / bm) * (a.N / band_cols(a)) <= 0x7fffffff)
+      return g == 8 ? launch_band<8>(a, bm, s) : (g == 4 ? launch_band<4>(a, bm, s) : launch_band<2>(a, bm, s));
+  }
   // the pipelined form: whole tiles (M, N, K are powers of two) for every SM,
   // two stages or more -- with a single stage there is nothing to overlap --
   // and 16-byte aligned operands

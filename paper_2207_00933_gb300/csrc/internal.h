@@ -189,21 +189,27 @@ cudaError_t gemm_simt_configure();   // one-time kernel attributes (dynamic shar
 
 constexpr int kOpThreads = 256;                  // threads of a contraction tile's or band's CTA
 // Bands of a step with a short shared index (gemm_band, device_ops.cuh).
-constexpr int kBandOutputs = 8192;               // outputs per band, as far as M allows
-constexpr int kBandSmemFloats = 2 * 4096 + 2 * 1024;
-__host__ __device__ inline int band_cols(int64_t N) { return N < 1024 ? int(N) : 1024; }
+constexpr int kBandOutputs = 16384;              // outputs per band, as far as M allows
+constexpr int kBandSmemFloats = 10240;
+__host__ __device__ inline int band_cols(const GemmArgs& a) {
+  const int most = a.K == 16 ? 256 : 512;
+  return a.N < most ? int(a.N) : most;
+}
 // Rows of a band of a step (0: the step does not take bands): `outputs` per
-// band or fewer.
+// band or fewer, whole groups of g rows (K = 16: of 8) for every row group of
+// threads, operands and offsets within kBandSmemFloats.
 inline int band_rows(const GemmArgs& a, int g, int64_t outputs) {
   if (!a.vec4 || a.kind != OUT_F32 || a.chunk > 0 || a.accumulate || a.N < 16) return 0;
   if (a.K != 1 && a.K != 4 && a.K != 16) return 0;
-  if ((reinterpret_cast<uintptr_t>(a.B) | reinterpret_cast<uintptr_t>(a.C)) & 15) return 0;
-  const int64_t bn = band_cols(a.N), least = int64_t(g) * (kOpThreads / (bn >> 2));
+  if ((reinterpret_cast<uintptr_t>(a.A) | reinterpret_cast<uintptr_t>(a.B) | reinterpret_cast<uintptr_t>(a.C)) & 15)
+    return 0;
+  const int64_t bn = band_cols(a), least = int64_t(a.K == 16 ? 8 : g) * (kOpThreads / (bn >> 2));
+  const int64_t most = a.K == 16 ? 256 : 1024;
   int64_t bm = outputs / bn;
-  if (bm > a.M) bm = a.M;
-  while (bm * a.K > 4096 || bm > 1024) bm >>= 1;
   if (bm < least) bm = least;
-  return bm <= a.M && bm * a.K <= 4096 && bm <= 1024 ? int(bm) : 0;
+  if (bm > a.M) bm = a.M;
+  if (bm > most) bm = most;
+  return bm >= least ? int(bm) : 0;
 }
 
 // ---- contraction step, split-BF16 on tcgen05 ---------------------------------
