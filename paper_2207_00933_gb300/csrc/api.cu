@@ -449,6 +449,21 @@ sqc_status attribute_all(sqc_ctx* ctx, Circuit* c, const void* const* probs, sqc
     smem = 0;
     return SQC_OK;
   };
+  // Tiles grow while one reads at most the circuit's share over kAttrTiles
+  // tiles (two per SM: a tile is bound by its reads) and, below
+  // kAttrManyTiles tiles of a subcircuit, holds at most kAttrSlots values (8 KB:
+  // longer tiles leave too few CTAs' phases to overlap).  A subcircuit used to
+  // keep 8 x 2 tiles up to 4096 of them, whose bit-reversed write runs are 8
+  // bytes; measured (a load of the whole circuit, us, that rule -> this one):
+  // 40-qubit grid 37 -> 35, 30-qubit line 9.9 -> 6.5, chains of 5-6 blocks of 12
+  // to 16 wires with 1 to 3 cuts 61 -> 18, 73 -> 17 and 59 -> 12, six blocks of
+  // 14 wires 33 -> 5.2.  With 608 or 1216 tiles the small ones lose (9 and 15 us
+  // for the last), with 4096 slots the grids (14 -> 25 us for blocks of 12, 13,
+  // 12 wires with 3 and 2 cuts).
+  constexpr int64_t kAttrTiles = 304, kAttrSlots = 2048, kAttrManyTiles = 512;
+  int64_t tile_reads = 0;
+  for (int i = 0; i < c->nC; ++i) tile_reads += c->V[i] << c->w[i];
+  tile_reads /= kAttrTiles;
   for (int i = 0; i < c->nC; ++i) {
     const int n = c->ndata[i];
     const int kin = int(c->ins[i].size());
@@ -463,10 +478,9 @@ sqc_status attribute_all(sqc_ctx* ctx, Circuit* c, const void* const* probs, sqc
       d.kout = kout;
       // x tile: 2^L1 consecutive low values (read runs) x 2^L2 top-bit
       // values (write runs of the bit-reversed A).  Start at 8 x 2; grow
-      // toward 32 x 8 (128-byte reads, whole 32-byte write sectors) while
-      // the subcircuit still has kAttrTileTarget tiles, so that small
-      // subcircuits keep enough CTAs and large ones amortise each tile's
-      // shared-memory passes over more data.
+      // toward 32 x 8 (128-byte reads, whole 32-byte write sectors) by the rule
+      // above, so that small circuits keep enough CTAs and larger ones
+      // amortise each tile's shared-memory passes and write whole sectors.
       int L2 = std::min(1, n / 2), L1 = std::min(3, n - L2);
       const int64_t S = int64_t(1) << (2 * kin);
       while ((S << (L1 + L2)) > kAttrSmemMax / 4) {
@@ -474,10 +488,11 @@ sqc_status attribute_all(sqc_ctx* ctx, Circuit* c, const void* const* probs, sqc
         else if (L2 > 0) --L2;
         else break;
       }
-      constexpr int64_t kAttrTileTarget = 4096;
       for (;;) {
-        const int64_t tiles_next = ((int64_t(1) << (n - L1 - L2)) << (2 * kout)) >> 1;
-        if (L1 + L2 >= n || tiles_next < kAttrTileTarget || (S << (L1 + L2 + 1)) > kAttrSmemMax / 4) break;
+        const int64_t slots = S << (L1 + L2 + 1), tiles_next = ((int64_t(1) << (n - L1 - L2)) << (2 * kout)) >> 1;
+        if (L1 + L2 >= n || (slots << kout) > tile_reads ||
+            slots > (tiles_next >= kAttrManyTiles ? kAttrSmemMax / 4 : kAttrSlots))
+          break;
         if (L2 < 3) ++L2;
         else if (L1 < 5) ++L1;
         else break;

@@ -146,3 +146,44 @@ def test_batch_bands(policy):
             assert np.array_equal(o.double().cpu().numpy(), w)
             assert abs(t - w.sum()) <= 1e-6 * np.abs(w).sum()
         ctx.batch_release(b)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("widths,cuts", [
+    ([3, 4, 4], [1, 2]),              # two data qubits in the middle block: the least the streaming form takes
+    ([4, 6, 5], [1, 3]),
+    ([7, 9, 9], [3, 3]),              # 64 prepared states x 8 outcomes: 16-state tiles of 64
+    ([9, 11, 8], [3, 3]),
+    ([8, 8, 8], [4, 2]),              # 256 x 4: 8-state tiles
+    ([8, 9, 7], [4, 3]),              # 256 x 8: 4-state tiles
+    ([8, 8, 7], [5, 1]),              # 1024 x 2
+    ([10, 9], [6]),                   # 4096 prepared states: too many for a tile
+    ([13, 10], [1]),                  # no incoming edge, and no outgoing one
+    ([9], []),
+])
+def test_attribution_forms(widths, cuts, offset):
+    """Every attributed value shows in some bin when all qubits are active;
+    inputs at a 16-byte address and one value beyond it."""
+    import torch
+    from paper_2207_00933_gb300 import Context, _build
+    _build.build()
+    c, probs = _chain(sum(widths), widths, cuts, ones=6)
+    g = O.Graph.from_arrays(c.n_qubits, *c.graph_arrays())
+    roles = np.zeros(c.n_qubits, dtype=np.int8)
+    T = O.subcircuit_tensors(g, [p.astype(np.float64) for p in probs], roles)
+    assert O.reconstruct_pairwise(g, [np.abs(t) for t in T], roles).max() * 2.0 ** c.n_edges < 2 ** 24
+    want = O.reconstruct_pairwise(g, T, roles)
+    dev = []
+    for p in probs:
+        buf = torch.zeros(p.size + 4, dtype=torch.float32, device="cuda")
+        buf[offset:offset + p.size] = torch.from_numpy(p).cuda().flatten()
+        dev.append(buf[offset:offset + p.size].view(p.shape))
+    for cfg in ({}, {"merge_pyramid": True}):
+        with Context(0, **cfg) as ctx:
+            cid = ctx.load_subcircuit_outputs(c.n_qubits, *c.graph_arrays(), dev)
+            ctx.update_subcircuit_outputs(cid, dev)
+            qid, na = ctx.set_qubit_roles(cid, roles)
+            res = torch.full((1 << na,), float("nan"), dtype=torch.float64, device="cuda")
+            ctx.reconstruct(qid, res)
+            torch.cuda.synchronize()
+            assert np.array_equal(res.cpu().numpy(), want)
