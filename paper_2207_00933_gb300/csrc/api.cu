@@ -557,11 +557,14 @@ sqc_status attribute_all(sqc_ctx* ctx, Circuit* c, const void* const* probs, sqc
   }
   sqc_status st = flush();
   if (st != SQC_OK) return st;
+  std::vector<PyramidDesc> pd;
   for (size_t i = 0; i < c->pyr.size(); ++i)
-    if (c->pyr[i]) {
-      CK(launch_pyramid(c->A[i], c->pyr[i], c->V[i], c->ndata[i], s));
-      ctx->launches += (c->ndata[i] + kPyramidLevelsPerPass - 1) / kPyramidLevelsPerPass;
-    }
+    if (c->pyr[i]) pd.push_back({c->A[i], c->pyr[i], c->V[i], c->ndata[i], 0, 0, 0});
+  if (!pd.empty()) {
+    int launches = 0;
+    CK(launch_pyramids(pd.data(), int(pd.size()), &launches, s));
+    ctx->launches += launches;
+  }
   if (!on_device) {
     // host inputs: the caller may reuse its buffers on return, except while
     // the stream is captured into a graph (no synchronisation is allowed

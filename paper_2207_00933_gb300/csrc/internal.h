@@ -160,11 +160,24 @@ inline bool merge_is_long(const MergeDesc& d) { return d.fast && d.lanes == 32 &
 cudaError_t launch_merge_blocks(const MergeDesc* descs, int n, int64_t total_blocks, bool tiled, cudaStream_t s);
 // The same for descriptors that are all merge_is_long, total_outputs of them
 cudaError_t launch_merge_long(const MergeDesc* descs, int n, int64_t total_outputs, cudaStream_t s);
-// Merge pyramid of one subcircuit (A: [V][2^n]): level m = 1..n at
+// Merge pyramid of a subcircuit (src = A: [V][2^n]): level m = 1..n at
 // pyr + V (2^n - 2^(n-m+1)), [V][2^(n-m)], level m = pairwise sums of level
-// m-1 (level 0 = A).  One launch per kPyramidLevelsPerPass levels.
+// m-1 (level 0 = A).  One launch per kPyramidLevelsPerPass levels for up to
+// kAttrPerLaunch subcircuits; s, c and block_begin are set by the launcher.
 constexpr int kPyramidLevelsPerPass = 10;
-cudaError_t launch_pyramid(const float* A, float* pyr, int64_t V, int n, cudaStream_t s);
+struct PyramidDesc {
+  const float* src;
+  float* pyr;
+  int64_t V;
+  int n;                     // levels in all
+  int s, c;                  // level read, and how many are made from it
+  int64_t block_begin;
+};
+struct PyramidLaunch {
+  PyramidDesc d[kAttrPerLaunch];
+  int n;
+};
+cudaError_t launch_pyramids(PyramidDesc* d, int n, int* launches, cudaStream_t s);
 
 // ---- contraction step, FP32 SIMT (Section 6.1: C = A B over the shared index)
 struct GemmArgs {
