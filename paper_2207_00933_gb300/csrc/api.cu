@@ -2366,6 +2366,26 @@ sqc_status reconstruct_stages(sqc_ctx* ctx, sqc_query_id qid, sqc_precision prec
       if (ms != SQC_OK) return ms;
     }
     for (size_t si = 0; si < P.steps.size(); ++si) {
+      // consecutive small steps before the last share a launch
+      {
+        SmallRun run{};
+        for (size_t sj = si; sj + 1 < P.steps.size() && run.n < kSmallRunMost; ++sj) {
+          const Step& t = P.steps[sj];
+          if (t.tc || !gemm_is_small(t.M, t.N, t.Kd)) break;
+          const Tensor& tz = P.tensors[t.z];
+          run.s[run.n++] = {static_cast<const float*>(P.tensors[t.x].buf), static_cast<const float*>(P.tensors[t.y].buf),
+                            t.rowmap, t.colmap, tz.buf, tz.plane_stride, static_cast<unsigned char>(ilog2(t.M)),
+                            static_cast<unsigned char>(ilog2(t.N)), static_cast<unsigned char>(ilog2(t.Kd)),
+                            static_cast<unsigned char>(tz.kind)};
+        }
+        if (run.n >= 2) {
+          StageScope scope(ctx, s, SQC_STAGE_CONTRACT);
+          CK(launch_gemm_small_run(run, s));
+          ctx->launches += 1;
+          si += size_t(run.n) - 1;
+          continue;
+        }
+      }
       const Step& st = P.steps[si];
       const bool last = int(si) == int(P.steps.size()) - 1;
       const Tensor& Z = P.tensors[st.z];

@@ -51,6 +51,60 @@ __global__ void __launch_bounds__(kPipeThreads, 3) gemm_pipe_kernel(GemmArgs a) 
   if (a.partials) finish_total(mysum, a.partials, a.counter, a.total, red);
 }
 
+// Steps of at most 1024 outputs and 16 shared terms, one after the other in
+// one CTA: what a long chain of narrow subcircuits contracts to (a 59-block
+// chain has 55 such steps in a row).  A launch each costs the host and the
+// GPU about 3 us; here a step is one round of loads from L2 (both operand
+// rows and the two map entries of an output together), its multiply-adds and
+// a store.  k runs upwards with gemm_tile's zero term below 16: the values are
+// the same bit for bit.  Bound: the latency of L2.
+__global__ void __launch_bounds__(kThreads) gemm_small_run_kernel(const __grid_constant__ SmallRun r) {
+  pdl_wait();      // the previous kernel on the stream has completed
+  pdl_trigger();   // the next one may start launching
+  for (int i = 0; i < r.n; ++i) {
+    const SmallStep& st = r.s[i];
+    const int nl = st.n_log2, outs = 1 << (st.m_log2 + nl), K = 1 << st.k_log2;
+    // every thread's offsets and operands before any store: an output's place
+    // may not depend on the step before, but its operands do
+    for (int o = threadIdx.x; o < outs; o += kThreads) {
+      const int row = o >> nl, col = o & ((1 << nl) - 1);
+      const uint64_t at = __ldg(st.rowmap + row) + __ldg(st.colmap + col);
+      float acc = 0.f;
+      if (K >= 4) {
+        const float4* a = reinterpret_cast<const float4*>(st.A + row * K);
+        const float4* b = reinterpret_cast<const float4*>(st.B + col * K);
+        if (K == 16) {
+          float4 x[4], y[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            x[q] = __ldcg(a + q);
+            y[q] = __ldcg(b + q);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            acc = fmaf(x[q].x, y[q].x, acc);
+            acc = fmaf(x[q].y, y[q].y, acc);
+            acc = fmaf(x[q].z, y[q].z, acc);
+            acc = fmaf(x[q].w, y[q].w, acc);
+          }
+        } else {
+          const float4 x = __ldcg(a), y = __ldcg(b);
+          acc = fmaf(x.x, y.x, acc);
+          acc = fmaf(x.y, y.y, acc);
+          acc = fmaf(x.z, y.z, acc);
+          acc = fmaf(x.w, y.w, acc);
+          acc = fmaf(0.f, 0.f, acc);
+        }
+      } else {
+        acc = fmaf(__ldcg(st.A + row), __ldcg(st.B + col), acc);
+        acc = fmaf(0.f, 0.f, acc);
+      }
+      store_out_f(st.C, st.kind, st.plane_stride, at, acc);
+    }
+    __syncthreads();
+  }
+}
+
 // Bands of a short shared index (gemm_band), one per CTA.
 template <int G>
 __global__ void __launch_bounds__(kThreads, 2) gemm_band_kernel(GemmArgs a, int bm) {
@@ -104,6 +158,11 @@ constexpr int64_t kBandLeast = int64_t(1) << 18;
 cudaError_t gemm_simt_configure() {
   return cudaFuncSetAttribute(gemm_pipe_kernel<128, 64, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               int(sizeof(float)) * gemm_pipe_smem_floats<128, 64>());
+}
+
+cudaError_t launch_gemm_small_run(const SmallRun& r, cudaStream_t s) {
+  if (r.n <= 0) return cudaSuccess;
+  return launch_k(gemm_small_run_kernel, dim3(1), dim3(kThreads), 0, s, false, r);
 }
 
 cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t s) {

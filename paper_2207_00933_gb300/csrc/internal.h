@@ -198,6 +198,25 @@ struct GemmArgs {
   double* total;
 };
 cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t s);
+// A run of consecutive small steps (gemm_is_small, FP32 or BF16-plane output,
+// unscaled) in one launch of one CTA, in order.
+constexpr int kSmallRunMost = 48;
+constexpr int kSmallOutputs = 1024;
+struct SmallStep {
+  const float* A;
+  const float* B;
+  const uint64_t* rowmap;
+  const uint64_t* colmap;
+  void* C;
+  int64_t plane_stride;
+  unsigned char m_log2, n_log2, k_log2, kind;
+};
+struct SmallRun {
+  SmallStep s[kSmallRunMost];
+  int n;
+};
+inline bool gemm_is_small(int64_t M, int64_t N, int64_t K) { return M * N <= kSmallOutputs && K <= 16; }
+cudaError_t launch_gemm_small_run(const SmallRun& r, cudaStream_t s);
 cudaError_t gemm_simt_configure();   // one-time kernel attributes (dynamic shared memory)
 
 constexpr int kOpThreads = 256;                  // threads of a contraction tile's or band's CTA
