@@ -220,19 +220,32 @@ template <int TM, int TN>
 __device__ __forceinline__ float store_tile_f32(const GemmArgs& a, const float (&acc)[TM][TN], int64_t row0,
                                                 int64_t c0, float alpha_f, void* Cout) {
   float sum_f = 0.f;
+  // every map entry before the first store: the compiler may not move a load
+  // over a store that might alias it, and one round trip per row is what the
+  // epilogue then takes
+  constexpr int kC = TN % 4 == 0 ? TN / 4 : TN;
+  uint64_t rb[TM], cb[kC];
+#pragma unroll
+  for (int i = 0; i < TM; ++i) rb[i] = row0 + i < a.M ? __ldg(a.rowmap + row0 + i) : 0;
+  const bool vec = a.vec4 && (TN % 4) == 0 && c0 + TN <= a.N;
+#pragma unroll
+  for (int j = 0; j < kC; ++j) {
+    const int64_t col = c0 + j * (TN / kC);
+    cb[j] = col < a.N ? __ldg(a.colmap + col) : 0;
+  }
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     const int64_t row = row0 + i;
     if (row >= a.M) continue;
-    const uint64_t rbase = a.rowmap[row];
-    if (a.vec4 && (TN % 4) == 0 && c0 + TN <= a.N) {
+    const uint64_t rbase = rb[i];
+    if (vec) {
 #pragma unroll
       for (int j = 0; j + 3 < TN; j += 4) {
         float4 q;
         q.x = acc[i][j] * alpha_f; q.y = acc[i][j + 1] * alpha_f;
         q.z = acc[i][j + 2] * alpha_f; q.w = acc[i][j + 3] * alpha_f;
         sum_f += (q.x + q.y) + (q.z + q.w);
-        float4* dst = reinterpret_cast<float4*>(static_cast<float*>(Cout) + rbase + a.colmap[c0 + j]);
+        float4* dst = reinterpret_cast<float4*>(static_cast<float*>(Cout) + rbase + cb[j / 4]);
         if (a.accumulate) {
           const float4 o = *dst;
           q.x += o.x; q.y += o.y; q.z += o.z; q.w += o.w;
@@ -246,7 +259,7 @@ __device__ __forceinline__ float store_tile_f32(const GemmArgs& a, const float (
         if (col >= a.N) continue;
         const float v = acc[i][j] * alpha_f;
         sum_f += v;
-        float* dst = static_cast<float*>(Cout) + rbase + a.colmap[col];
+        float* dst = static_cast<float*>(Cout) + rbase + (kC == TN ? cb[j < kC ? j : 0] : __ldg(a.colmap + col));
         *dst = a.accumulate ? *dst + v : v;
       }
     }
@@ -372,11 +385,16 @@ __device__ __forceinline__ double gemm_tile(const GemmArgs& a, int64_t m0, int64
     if (a.kind == OUT_F32) return double(store_tile_f32<TM, TN>(a, acc, m0 + ty * TM, n0 + tx * TN, alpha_f, Cout));
   float sum_f = 0.f;
   double sum_d = 0.0;
+  uint64_t rb[TM], cb[TN];                 // map entries before any store, as above
+#pragma unroll
+  for (int i = 0; i < TM; ++i) rb[i] = m0 + ty * TM + i < a.M ? __ldg(a.rowmap + m0 + ty * TM + i) : 0;
+#pragma unroll
+  for (int j = 0; j < TN; ++j) cb[j] = n0 + tx * TN + j < a.N ? __ldg(a.colmap + n0 + tx * TN + j) : 0;
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     const int64_t row = m0 + ty * TM + i;
     if (row >= a.M) continue;
-    const uint64_t rbase = a.rowmap[row];
+    const uint64_t rbase = rb[i];
     const int64_t c0 = n0 + tx * TN;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
@@ -386,13 +404,13 @@ __device__ __forceinline__ double gemm_tile(const GemmArgs& a, int64_t m0, int64
       if constexpr (CHUNKED) v = acc64[i][j]; else v = f2d(acc[i][j] * alpha_f);
       if (a.kind == OUT_F64) sum_d += v; else sum_f += float(v);
       if (a.accumulate && a.kind == OUT_F64) {
-        double* dst = static_cast<double*>(Cout) + rbase + a.colmap[col];
+        double* dst = static_cast<double*>(Cout) + rbase + cb[j];
         *dst += v;                          // slices add up in FP64
       } else if (a.accumulate && a.kind == OUT_F32) {
-        float* dst = static_cast<float*>(Cout) + rbase + a.colmap[col];
+        float* dst = static_cast<float*>(Cout) + rbase + cb[j];
         *dst += float(v);
       } else {
-        store_out(Cout, a.kind, a.plane_stride, rbase + a.colmap[col], v);
+        store_out(Cout, a.kind, a.plane_stride, rbase + cb[j], v);
       }
     }
   }

@@ -1053,6 +1053,11 @@ __device__ __noinline__ void tail_tile_apart(const GemmArgs& a, int64_t m0, int6
   gemm_tile<BM, BM, TMN, TMN, false, BK, kRThreads, true>(a, m0, n0, stage, stage + BK * (BM + 4), a.C);
 }
 
+// The same for 32 x 32 tiles beyond tail_tile32 (a long shared index).
+__device__ __noinline__ void tail_tile32_long(const GemmArgs& a, int64_t m0, int64_t n0, float* stage) {
+  gemm_tile<32, 32, 1, 1, false, 64, kRThreads, true>(a, m0, n0, stage, stage + 64 * (32 + 4), a.C);
+}
+
 // A 32 x 32 tile of an FP32 step with K <= 64 on the whole CTA, one output
 // per thread: both operand tiles and the output's two layout-map entries
 // are loaded in one round (the general tile loads A, then B, then reads the
@@ -1126,7 +1131,7 @@ __device__ __forceinline__ bool tail_pre_steps(const TailArgs& T, ResWork& w, un
       if (ts.cfg == 0 && a.K <= 64 && a.kind == OUT_F32)
         tail_tile32(a, m0, n0, stage);
       else if (ts.cfg == 0)
-        gemm_tile<32, 32, 1, 1, false, 64, kRThreads, true>(a, m0, n0, stage, stage + 64 * (32 + 4), a.C);
+        tail_tile32_long(a, m0, n0, stage);
       else if (ts.cfg == 1)
         tail_tile_apart<64, 2, 32>(a, m0, n0, stage);
       else
