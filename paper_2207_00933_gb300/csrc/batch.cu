@@ -1,19 +1,24 @@
 // Batched recursion level: many queries (bins of possibly different
-// circuits, uneven active-qubit counts) reconstructed by ONE persistent
-// kernel launch.
+// circuits, uneven active-qubit counts) reconstructed together: the merges of
+// all of them in one launch, then their contraction steps in one persistent
+// launch.  (A single query's one launch keeps its merges in the work list.)
 //
-// The host flattens every query's merge blocks and contraction-step tiles
-// into one work list ordered by dependency level (all merge blocks first,
-// then the steps level by level).  Persistent CTAs take items in list order
-// from a global head counter.  Every tensor has a completion counter; an
-// item waits (bounded) until the counters of its input tensors reach their
-// expected item counts, does its work, then bumps the counter of the tensor
-// it wrote.  An item only ever waits for items earlier in the list, which
-// were taken by CTAs that are running, so the schedule cannot deadlock.
-// The last CTA to leave re-arms the head and the counters, so the same
-// launch can be replayed (e.g. from a CUDA graph).  On a wait timeout the
-// kernel raises an abort flag that makes every CTA drain quickly and
-// records an error code.
+// The host flattens every query's contraction bands and tiles into one work
+// list ordered by dependency level.  Persistent CTAs claim items in list order
+// from a global head counter, one ahead of the item they work on.  Every
+// tensor has a completion counter; an item waits (bounded) until the counters
+// of its input tensors reach their expected item counts, does its work, then
+// bumps the counter of the tensor it wrote.  An item only ever waits for items
+// earlier in the list, and every CTA works through its claims in order, so the
+// earliest unfinished item always runs and the schedule cannot deadlock.  The
+// last CTA to leave re-arms the head and the counters, so the same launch can
+// be replayed (e.g. from a CUDA graph).  On a wait timeout the kernel raises
+// an abort flag that makes every CTA drain quickly and records an error code.
+//
+// Bound: the latency of its items (operands, map entries and counters from
+// L2).  256 queries of 10 to 20 active qubits over four circuits (165 MB of
+// bins, 863 MB of states merged from L2): 180 us, 66 of them the merges, where
+// one launch with a merge block or a 32 x 32 tile per item took 833 us.
 #include "device_ops.cuh"
 
 namespace sqc {
