@@ -1670,7 +1670,7 @@ sqc_status build_batch(sqc_ctx* ctx, int32_t n, Query* const* qv, void* const* o
     dev_free(ctx, B->work, B->work_bytes);
     return cuda_fail(ctx, e, "batch upload");
   }
-  int sms = 152, per = 2;
+  int sms = 152, per = 3;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   B->phases.assign(n_phases, BatchLaunch{});
   B->phase_grid.assign(n_phases, 0);

@@ -16,9 +16,12 @@
 // an abort flag that makes every CTA drain quickly and records an error code.
 //
 // Bound: the latency of its items (operands, map entries and counters from
-// L2).  256 queries of 10 to 20 active qubits over four circuits (165 MB of
-// bins, 863 MB of states merged from L2): 180 us, 66 of them the merges, where
-// one launch with a merge block or a 32 x 32 tile per item took 833 us.
+// L2), so three CTAs per SM although the 64 x 64 tiles then spill.  256 queries
+// of 10 to 20 active qubits over four circuits (165 MB of bins, 863 MB of
+// states merged from L2): 162 us, 66 of them the merges (180 with two CTAs per
+// SM, 158 with four, where longer shared indices lose: 64 queries of K = 64
+// steps 210, 197 and 200 us); one launch with a merge block or a 32 x 32 tile
+// per item took 833 us.
 #include "device_ops.cuh"
 
 namespace sqc {
@@ -74,7 +77,7 @@ __device__ __forceinline__ double run_tile(const BatchStep& st, int64_t tile, fl
   return gemm_tile<BM, BN, TM, TN, CH, BK, kOpThreads, true>(st.a, m0, n0, smem, smem + BK * (BM + 4), C);
 }
 
-__global__ void __launch_bounds__(kOpThreads, 2) batch_kernel(BatchLaunch L) {
+__global__ void __launch_bounds__(kOpThreads, 3) batch_kernel(BatchLaunch L) {
   pdl_wait();      // the previous kernel on the stream has completed
   pdl_trigger();   // the next one may start launching
   extern __shared__ __align__(16) float smem[];
