@@ -364,6 +364,12 @@ size_t select_resident_smem(uint64_t n, int is_f64, int grid, uint64_t* per);
 cudaError_t launch_select_resident(void* work, int grid, const void* x, int is_f64, uint64_t n, int k,
                                    double threshold, unsigned long long* bins_out, double* probs_out, int* n_found,
                                    int* err, cudaStream_t s);
+// The same selection by one CTA, without a workspace: at most kSmallMost values
+// and kSmallMaxK bins.
+constexpr uint64_t kSmallMost = 4096;
+constexpr int kSmallMaxK = 128;
+cudaError_t launch_select_small(const void* x, int is_f64, uint64_t n, int k, double threshold,
+                                unsigned long long* bins_out, double* probs_out, int* n_found, cudaStream_t s);
 // The same selection for inputs of any size, read once: a sample bounds the
 // k-th value from below and only the values above the bound are kept.  Same
 // workspace, grid = select_resident_grid() (> 0).  Up to kStreamMost values
