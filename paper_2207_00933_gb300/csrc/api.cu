@@ -2099,8 +2099,9 @@ sqc_status select_bins(sqc_ctx* ctx, Query& q, const void* probs, bool is_f64, u
   // has no sample to take (2^20 FP32 values 15-20 us against 22-25 us, 2^22
   // 22-30 against 24-25), but holds and counts every value where the
   // filtering form touches each once (6.3 M FP32 values 28-39 us against
-  // 25-27, FP64 45-55 against 38-49).  Up to kSmallMost values and kSmallMaxK
-  // bins one CTA without grid barriers: 4-10 us against 12-14.
+  // 25-27; FP64 2^22 25-32, 6.3 M in the filtering form 38-49).  Up to
+  // kSmallMost values and kSmallMaxK bins one CTA without grid barriers: 4-10
+  // us against 12-14.
   constexpr uint64_t kResidentMost = uint64_t(5) << 20;
   if (rgrid > 0 && ctx->cfg.select_resident && n <= kSmallMost && r.k <= kSmallMaxK)
     CK(launch_select_small(probs, is_f64, n, r.k, r.threshold, r.bins, r.probs, r.n_found, s));

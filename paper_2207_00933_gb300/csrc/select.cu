@@ -1503,7 +1503,12 @@ struct StreamArgs {
   CoopWork coop;              // workspace and
   int coop_cap;               // bucket capacity of the fallback
 };
-struct NoSource {};
+// Vectors per thread on their way through shared memory in the resident form's
+// load of its slice (four are no faster, and three fit beside 5 M values).
+constexpr int kLoadRing = 3;
+struct NoSource {
+  int ring;                    // whether shared memory holds the ring beside the slice's keys
+};
 
 // The sampled chunk of stratum s: a fixed pseudo-random multiple of 4 inside
 // it (a mixing function of the index, so that no period of the input lines
@@ -2007,52 +2012,67 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
       if (lane == 0 && T.total) T.partials[blockIdx.x] = double(h) + double(l);
     }
   } else {
-    // the loop bound is the same for the whole CTA: warp_hist_add needs
-    // every lane of the warp
-    for (int b0 = 0; b0 < cnt; b0 += kRThreads * V) {
-      const int i0 = b0 + tid * V;
-      unsigned kv[V];
-      if constexpr (F64) {
-        const double* p = static_cast<const double*>(x) + start + i0;
-        double a[2];
-        if (aligned && i0 + 2 <= cnt) {
-          const double2 q = __ldg(reinterpret_cast<const double2*>(p));
+    // The slice's vectors go through each thread's own slots of a ring
+    // (cp.async, kLoadRing - 1 rounds ahead, no barrier): one CTA per SM is
+    // bound by the loads in flight, and plain loads by the small L1 that is
+    // left beside this much shared memory (2^22 FP64 values from L2, the whole
+    // selection: 35-42 us with plain loads, 25-32 us so; FP32 the same).  The
+    // loop bound is the same for the whole CTA: warp_hist_add needs every lane
+    // of the warp.
+    using Word = std::conditional_t<F64, unsigned long long, unsigned>;
+    unsigned char* ring = reinterpret_cast<unsigned char*>(keys + per);
+    const bool ringed = aligned && T.ring;
+    const int vecs = cnt / V;
+    auto request = [&](int r) {
+      const int v = r * kRThreads + tid;
+      if (v < vecs)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(uint32_t(__cvta_generic_to_shared(
+                         ring + (size_t(r % kLoadRing) * kRThreads + tid) * 16))),
+                     "l"(static_cast<const Word*>(x) + start + size_t(v) * V)
+                     : "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (ringed)
+      for (int r = 0; r < kLoadRing - 1; ++r) request(r);
+    for (int r = 0; r * kRThreads * V < cnt; ++r) {
+      const int i0 = (r * kRThreads + tid) * V;
+      Word a[V];
+      if (ringed) {
+        request(r + kLoadRing - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kLoadRing - 1) : "memory");
+      }
+      if (aligned && i0 + V <= cnt) {
+        const void* from = ringed ? static_cast<const void*>(ring + (size_t(r % kLoadRing) * kRThreads + tid) * 16)
+                                  : static_cast<const void*>(static_cast<const Word*>(x) + start + i0);
+        if constexpr (F64) {
+          const ulonglong2 q = *static_cast<const ulonglong2*>(from);
           a[0] = q.x; a[1] = q.y;
         } else {
-          a[0] = i0 < cnt ? p[0] : __longlong_as_double(0x7ff8000000000000ll);
-          a[1] = i0 + 1 < cnt ? p[1] : __longlong_as_double(0x7ff8000000000000ll);
-        }
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const unsigned long long u = __double_as_longlong(a[q]);
-          const bool nan = (u & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
-          const unsigned long long kk = key_f64(a[q]);
-          kv[q] = (!nan && kk >= key_thr) ? unsigned(kk >> 32) : 0u;
+          const uint4 q = *static_cast<const uint4*>(from);
+          a[0] = q.x; a[1] = q.y; a[2] = q.z; a[3] = q.w;
         }
       } else {
-        const float* p = static_cast<const float*>(x) + start + i0;
-        float a[4];
-        if (aligned && i0 + 4 <= cnt) {
-          const float4 q = __ldg(reinterpret_cast<const float4*>(p));
-          a[0] = q.x; a[1] = q.y; a[2] = q.z; a[3] = q.w;
-        } else {
+        const Word none = F64 ? Word(0x7ff8000000000000ull) : Word(0x7fc00000u);      // NaN
 #pragma unroll
-          for (int q = 0; q < 4; ++q) a[q] = i0 + q < cnt ? p[q] : __uint_as_float(0x7fc00000u);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const unsigned u = __float_as_uint(a[q]);
-          const bool nan = (u & 0x7fffffffu) > 0x7f800000u;
-          const unsigned kk = unsigned(key_f32(a[q]) >> 32);
-          kv[q] = (!nan && kk >= unsigned(key_thr)) ? kk : 0u;
-        }
+        for (int q = 0; q < V; ++q) a[q] = i0 + q < cnt ? static_cast<const Word*>(x)[start + i0 + q] : none;
       }
 #pragma unroll
       for (int q = 0; q < V; ++q) {
-        if (i0 + q < cnt) keys[i0 + q] = kv[q];
-        warp_hist_add(sh, kv[q] != 0, kv[q] >> (32 - kRBits), lane);
+        unsigned kv;
+        if constexpr (F64) {
+          const bool nan = (a[q] & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
+          const unsigned long long kk = key_f64(__longlong_as_double((long long)a[q]));
+          kv = (!nan && kk >= key_thr) ? unsigned(kk >> 32) : 0u;
+        } else {
+          const bool nan = (a[q] & 0x7fffffffu) > 0x7f800000u;
+          const unsigned kk = unsigned(key_f32(__uint_as_float(a[q])) >> 32);
+          kv = (!nan && kk >= unsigned(key_thr)) ? kk : 0u;
+        }
+        if (i0 + q < cnt) keys[i0 + q] = kv;
+        warp_hist_add(sh, kv != 0, kv >> (32 - kRBits), lane);
       }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
   // STREAM: what the CTAs' filters found, read after the first barrier;
   // false: the filter's result cannot be used
@@ -2541,8 +2561,15 @@ cudaError_t launch_select_resident(void* work, int grid, const void* x, int is_f
                                    int* err, cudaStream_t s) {
   if (k < 1 || k > kSelectMaxK) return cudaErrorInvalidValue;
   uint64_t per = 0;
-  const size_t smem = select_resident_smem(n, is_f64, grid, &per);
+  size_t smem = select_resident_smem(n, is_f64, grid, &per);
   if (!smem) return cudaErrorInvalidValue;
+  // no ring for a slice of one round
+  NoSource src{};
+  const size_t with_ring = size_t(kRHistBytes) + per * 4 + size_t(kLoadRing) * kRThreads * 16;
+  if (per > uint64_t(kRThreads) * (is_f64 ? 2 : 4) && with_ring <= size_t(kRSmemMax)) {
+    src.ring = 1;
+    if (smem < with_ring) smem = with_ring;
+  }
   // refinement stops once the k-th value's bucket holds at most cap values:
   // the values above it (< k) and the bucket then fit the ranking's
   // kMaxSort candidates, which costs less than another digit pass and its
@@ -2551,12 +2578,11 @@ cudaError_t launch_select_resident(void* work, int grid, const void* x, int is_f
   ResWork w = resident_work(work);
   const int aligned = (reinterpret_cast<uintptr_t>(x) % 16) == 0;
   const unsigned long long kt = threshold_key(is_f64, threshold);
-  const NoSource none{};
   if (is_f64)
     return launch_k(select_resident_kernel<true, NoSource>, dim3(grid), dim3(kRThreads), smem, s, true, x, aligned, n,
-                    per, kt, k, cap, w, bins_out, probs_out, n_found, err, none);
+                    per, kt, k, cap, w, bins_out, probs_out, n_found, err, src);
   return launch_k(select_resident_kernel<false, NoSource>, dim3(grid), dim3(kRThreads), smem, s, true, x, aligned, n,
-                  per, kt, k, cap, w, bins_out, probs_out, n_found, err, none);
+                  per, kt, k, cap, w, bins_out, probs_out, n_found, err, src);
 }
 
 cudaError_t launch_select_small(const void* x, int is_f64, uint64_t n, int k, double threshold,
