@@ -37,6 +37,7 @@ constexpr int kMaxSub = 64;
 // Most outputs of a query merged by one warp each in small CTAs
 // (launch_merge_long): beyond, the plain kernel has warps enough.
 constexpr int64_t kMergeLongMost = 8192;
+constexpr int kMergeLongApart = 14;   // log2 of the run from which they leave the others' launch
 
 struct Circuit {
   int n_qubits = 0, nC = 0, K = 0;
@@ -1241,10 +1242,20 @@ sqc_status finalize_plan(sqc_ctx* ctx, Plan* P) {
     P->steps[s].rowmap = maps_dev + D.step_map_off[s].first;
     P->steps[s].colmap = maps_dev + D.step_map_off[s].second;
   }
+  // Few outputs over long runs, a warp per output: a query's whole merge when
+  // every subcircuit's is (merge_is_long), else a launch of its own for those of
+  // 2^14 states and more, whose warps would outlast the others by more than the
+  // launch costs (8 outputs of 2^19 states beside others: the merge 570-850 us,
+  // 157 so).
   int64_t blocks = 0, long_outputs = 0;
-  bool all_long = true, any_tiled = false;
+  bool any_tiled = false, all_long = true;
+  for (const MergeDesc& d : P->merge_host) all_long = all_long && merge_is_long(d);
+  auto by_warps = [&](const MergeDesc& d) { return merge_is_long(d) && (all_long || d.m >= kMergeLongApart); };
+  for (const MergeDesc& d : P->merge_host) long_outputs += by_warps(d) ? d.rows << d.a : 0;
+  if (long_outputs > kMergeLongMost) long_outputs = 0;
   for (int i = 0; i < nC; ++i) {
     MergeDesc& d = P->merge_host[i];
+    d.warps = long_outputs > 0 && by_warps(d);
     d.rowmap = maps_dev + D.merge_map_off[i].first;
     d.colmap = maps_dev + D.merge_map_off[i].second;
     d.dst = P->tensors[i].buf;          // null for the result (set per call)
@@ -1271,14 +1282,12 @@ sqc_status finalize_plan(sqc_ctx* ctx, Plan* P) {
                 int(lay.size()) > 0 && i != P->final_tensor;
     }
     d.block_begin = blocks;
-    blocks += merge_blocks_of(d);
-    long_outputs += d.rows << d.a;
-    all_long = all_long && merge_is_long(d);
+    if (!d.warps) blocks += merge_blocks_of(d);
     any_tiled = any_tiled || d.tiled;
   }
   P->merge_blocks = blocks;
   P->merge_tiled = any_tiled;
-  P->merge_long = all_long && long_outputs <= kMergeLongMost ? long_outputs : 0;
+  P->merge_long = long_outputs;
   cudaError_t e = upload(ctx, maps_dev, D.maps.data(), sizeof(uint64_t) * D.maps.size());
   if (e == cudaSuccess && nC > 0) {
     // one descriptor set per slice: slice sigma fixes sliced edge j's digit
@@ -2303,9 +2312,14 @@ sqc_status reconstruct_stages(sqc_ctx* ctx, sqc_query_id qid, sqc_precision prec
       }
       return SQC_OK;
     }
-    if (P.merge_long > 0) CK(launch_merge_long(descs, nd, P.merge_long, s));
-    else CK(launch_merge_blocks(descs, nd, P.merge_blocks, P.merge_tiled, s));
-    ctx->launches += 1;
+    if (P.merge_long > 0) {
+      CK(launch_merge_long(descs, nd, P.merge_long, s));
+      ctx->launches += 1;
+    }
+    if (P.merge_blocks > 0) {
+      CK(launch_merge_blocks(descs, nd, P.merge_blocks, P.merge_tiled, s));
+      ctx->launches += 1;
+    }
     return SQC_OK;
   };
 

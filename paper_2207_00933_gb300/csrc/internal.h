@@ -127,6 +127,7 @@ struct MergeDesc {
   int fast;                               // mer_mask == low m bits, act_mask == next a bits
   int lanes;                              // threads cooperating on one output (1..32, pow2)
   int tiled;                              // outputs transposed through shared memory (merge_tile)
+  int warps;                              // merged by launch_merge_long, not by launch_merge_blocks
   unsigned char rowbit[32];               // bit of the row index at the j-th lowest destination position
   const uint64_t* rowmap;                 // [rows]
   const uint64_t* colmap;                 // [2^a]
@@ -158,7 +159,7 @@ inline bool merge_is_long(const MergeDesc& d) { return d.fast && d.lanes == 32 &
 // descs: device array of n descriptors; total_blocks = CTAs over all of them;
 // tiled: some descriptor is
 cudaError_t launch_merge_blocks(const MergeDesc* descs, int n, int64_t total_blocks, bool tiled, cudaStream_t s);
-// The same for descriptors that are all merge_is_long, total_outputs of them
+// The same for the descriptors marked `warps`, total_outputs of them
 cudaError_t launch_merge_long(const MergeDesc* descs, int n, int64_t total_outputs, cudaStream_t s);
 // Merge pyramid of a subcircuit (src = A: [V][2^n]): level m = 1..n at
 // pyr + V (2^n - 2^(n-m+1)), [V][2^(n-m)], level m = pairwise sums of level

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(32 * kLongWarps) merge_long_kernel(const Merge
   if (o >= total) return;
   int i = 0;
   for (; i + 1 < n; ++i) {                        // the descriptor that holds output o
-    const int64_t cnt = descs[i].rows << descs[i].a;
+    const int64_t cnt = descs[i].warps ? descs[i].rows << descs[i].a : 0;
     if (o < cnt) break;
     o -= cnt;
   }

@@ -108,6 +108,17 @@ def test_long_merge(widths, cuts, active, zoom):
         _check(c, probs, W.lowest_active_roles(c, active, zoom), out=out)
 
 
+@pytest.mark.parametrize("widths,cuts,active", [
+    ([18, 6], [1], [2, 5]), ([6, 18], [1], [4, 3]), ([6, 18, 7], [1, 1], [3, 2, 5]),
+    ([17, 5, 18], [1, 1], [2, 2, 3]), ([16, 6], [1], [2, 5]), ([15, 6], [1], [0, 4])])
+def test_long_merge_beside_others(widths, cuts, active):
+    """Runs of 2^13 to 2^15 states, in each place among subcircuits of short
+    ones: merged in a launch of their own from 2^14 on."""
+    c, probs = _chain(7 + sum(widths), widths, cuts, ones=40)
+    for out in ("float32", "float64"):
+        _check(c, probs, W.lowest_active_roles(c, active), out=out)
+
+
 @pytest.mark.parametrize("policy", [0, 2])
 def test_batch_bands(policy):
     """The batched launch's bands (shared index 1, 4 and 16, from the smallest
