@@ -215,11 +215,14 @@ __device__ __forceinline__ float ld_operand(const float* p) {
 }
 
 // A thread's TM x TN FP32 outputs (first row row0, first column c0), scaled and
-// written through the layout maps; returns their FP32 sum.
-template <int TM, int TN>
-__device__ __forceinline__ float store_tile_f32(const GemmArgs& a, const float (&acc)[TM][TN], int64_t row0,
-                                                int64_t c0, float alpha_f, void* Cout) {
-  float sum_f = 0.f;
+// written through the layout maps; returns the FP64 sum of the FP32 sums of its
+// GR x GC groups.
+template <int TM, int TN, int GR = TM, int GC = TN>
+__device__ __forceinline__ double store_tile_f32(const GemmArgs& a, const float (&acc)[TM][TN], int64_t row0,
+                                                 int64_t c0, float alpha_f, void* Cout) {
+  static_assert(TM % GR == 0 && TN % GC == 0 && (GC == TN || GC % 4 == 0), "whole groups");
+  double sum = 0.0;
+  float group[TN / GC] = {};
   // every map entry before the first store: the compiler may not move a load
   // over a store that might alias it, and one round trip per row is what the
   // epilogue then takes
@@ -235,16 +238,16 @@ __device__ __forceinline__ float store_tile_f32(const GemmArgs& a, const float (
   }
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
-    const int64_t row = row0 + i;
-    if (row >= a.M) continue;
     const uint64_t rbase = rb[i];
-    if (vec) {
+    if (row0 + i >= a.M) {
+      // (no such row)
+    } else if (vec) {
 #pragma unroll
       for (int j = 0; j + 3 < TN; j += 4) {
         float4 q;
         q.x = acc[i][j] * alpha_f; q.y = acc[i][j + 1] * alpha_f;
         q.z = acc[i][j + 2] * alpha_f; q.w = acc[i][j + 3] * alpha_f;
-        sum_f += (q.x + q.y) + (q.z + q.w);
+        group[j / GC] += (q.x + q.y) + (q.z + q.w);
         float4* dst = reinterpret_cast<float4*>(static_cast<float*>(Cout) + rbase + cb[j / 4]);
         if (a.accumulate) {
           const float4 o = *dst;
@@ -258,13 +261,20 @@ __device__ __forceinline__ float store_tile_f32(const GemmArgs& a, const float (
         const int64_t col = c0 + j;
         if (col >= a.N) continue;
         const float v = acc[i][j] * alpha_f;
-        sum_f += v;
+        group[j / GC] += v;
         float* dst = static_cast<float*>(Cout) + rbase + (kC == TN ? cb[j < kC ? j : 0] : __ldg(a.colmap + col));
         *dst = a.accumulate ? *dst + v : v;
       }
     }
+    if ((i + 1) % GR == 0) {
+#pragma unroll
+      for (int j = 0; j < TN / GC; ++j) {
+        sum += double(group[j]);
+        group[j] = 0.f;
+      }
+    }
   }
-  return sum_f;
+  return sum;
 }
 
 // One BM x BN tile (origin m0, n0) of C = A B^T (Section 6.1) on NT threads
@@ -382,7 +392,7 @@ __device__ __forceinline__ double gemm_tile(const GemmArgs& a, int64_t m0, int64
   // FP32 outputs are scaled and summed in FP32; only FP64 outputs use the
   // FP64 pipe per element
   if constexpr (!CHUNKED)
-    if (a.kind == OUT_F32) return double(store_tile_f32<TM, TN>(a, acc, m0 + ty * TM, n0 + tx * TN, alpha_f, Cout));
+    if (a.kind == OUT_F32) return store_tile_f32<TM, TN>(a, acc, m0 + ty * TM, n0 + tx * TN, alpha_f, Cout);
   float sum_f = 0.f;
   double sum_d = 0.0;
   uint64_t rb[TM], cb[TN];                 // map entries before any store, as above
@@ -431,7 +441,10 @@ __device__ __forceinline__ void fma2(float2& d, float2 a, float2 b) {
 // A during the first half of the current stage and B during the second, into
 // the other shared-memory buffer (one CTA barrier per stage), and the
 // multiply-adds are issued two columns at a time.  k runs upwards as in
-// gemm_tile, so the values are the same bit for bit.  B's columns lie in
+// gemm_tile, so the values are the same bit for bit.  The probability check's
+// FP32 groups are G x G outputs, those of the plain tile in its place: 4 x 4
+// where 64 x 64 tiles would run (2^21 outputs: 128 tiles of 128 x 128 are too
+// few), 8 x 8 beyond.  B's columns lie in
 // shared memory with the two float4 halves of a thread's 8 columns apart, so
 // that a warp's 16-byte reads do not collide.  128 threads with 8 x 8 outputs
 // each, three CTAs per SM.  (Measured and not kept: 16 x 8 outputs a thread,
@@ -447,7 +460,7 @@ constexpr int gemm_pipe_smem_floats() {
   return 2 * kPipeK * (BM + 4 + BN + 4);
 }
 constexpr int kPipeThreads = 128;
-template <int BM, int BN, int TM, int TN, bool CG = false>
+template <int BM, int BN, int TM, int TN, int G, bool CG = false>
 __device__ __forceinline__ double gemm_tile_pipe(const GemmArgs& a, int64_t m0, int64_t n0, float* smem,
                                                  void* Cout) {
   constexpr int NT = kPipeThreads, TX = BN / TN;
@@ -536,13 +549,8 @@ __device__ __forceinline__ double gemm_tile_pipe(const GemmArgs& a, int64_t m0, 
     __syncthreads();
     cur ^= 1;
   }
-  // (the probability check's FP32 groups: 8 rows, as gemm_tile's)
-  double sum = 0.0;
-#pragma unroll
-  for (int i = 0; i < TM; i += 8)
-    sum += double(store_tile_f32<8, TN>(a, reinterpret_cast<const float(&)[8][TN]>(acc[i]), m0 + ty * TM + i,
-                                        n0 + tx * TN, pow2_to_float(a.alpha), Cout));
-  return sum;
+  return store_tile_f32<TM, TN, G, G>(a, reinterpret_cast<const float(&)[TM][TN]>(acc), m0 + ty * TM, n0 + tx * TN,
+                                      pow2_to_float(a.alpha), Cout);
 }
 
 

@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(GemmArgs a) {
   if (a.partials) finish_total(mysum, a.partials, a.counter, a.total, red);
 }
 
-template <int BM, int BN, int TM, int TN>
+template <int BM, int BN, int TM, int TN, int G>
 __global__ void __launch_bounds__(kPipeThreads, 3) gemm_pipe_kernel(GemmArgs a) {
   pdl_wait();      // the previous kernel on the stream has completed
   pdl_trigger();   // the next one may start launching
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kPipeThreads, 3) gemm_pipe_kernel(GemmArgs a) 
   const int64_t tile = blockIdx.x;
   const int64_t m0 = (tile >> tn_shift) * BM;
   const int64_t n0 = (tile & ((int64_t(1) << tn_shift) - 1)) * BN;
-  const double mysum = gemm_tile_pipe<BM, BN, TM, TN>(a, m0, n0, smem, a.C);
+  const double mysum = gemm_tile_pipe<BM, BN, TM, TN, G>(a, m0, n0, smem, a.C);
   if (a.partials) finish_total(mysum, a.partials, a.counter, a.total, red);
 }
 
@@ -126,9 +126,9 @@ cudaError_t launch_band(const GemmArgs& a, int bm, cudaStream_t s) {
                   false, a, bm);
 }
 
-template <int BM, int BN, int TM, int TN>
+template <int BM, int BN, int TM, int TN, int G>
 cudaError_t launch_pipe(const GemmArgs& a, cudaStream_t s) {
-  return launch_k(gemm_pipe_kernel<BM, BN, TM, TN>, dim3(unsigned((a.M / BM) * (a.N / BN))), dim3(kPipeThreads),
+  return launch_k(gemm_pipe_kernel<BM, BN, TM, TN, G>, dim3(unsigned((a.M / BM) * (a.N / BN))), dim3(kPipeThreads),
                   sizeof(float) * gemm_pipe_smem_floats<BM, BN>(), s, false, a);
 }
 
@@ -156,8 +156,11 @@ constexpr int64_t kBandLeast = int64_t(1) << 18;
 }
 
 cudaError_t gemm_simt_configure() {
-  return cudaFuncSetAttribute(gemm_pipe_kernel<128, 64, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(sizeof(float)) * gemm_pipe_smem_floats<128, 64>());
+  constexpr int smem = int(sizeof(float)) * gemm_pipe_smem_floats<128, 64>();
+  const cudaError_t e =
+      cudaFuncSetAttribute(gemm_pipe_kernel<128, 64, 8, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(gemm_pipe_kernel<128, 64, 8, 8, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 cudaError_t launch_gemm_small_run(const SmallRun& r, cudaStream_t s) {
@@ -189,7 +192,7 @@ cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t s) {
   const int64_t pipe_tiles = (a.M / 128) * (a.N / 64);
   if (wide && a.K >= 2 * kPipeK && pipe_tiles >= want && pipe_tiles <= 0x7fffffff &&
       ((reinterpret_cast<uintptr_t>(a.A) | reinterpret_cast<uintptr_t>(a.B)) & 15) == 0)
-    return launch_pipe<128, 64, 8, 8>(a, s);
+    return tiles(128, 128) >= want ? launch_pipe<128, 64, 8, 8, 8>(a, s) : launch_pipe<128, 64, 8, 8, 4>(a, s);
   if (wide && tiles(128, 128) >= want) return launch_cfg<128, 128, 8, 8, false>(a, s);
   if (!wide && tiles(128, 64) >= want) {
     if (chunked) return launch_cfg<128, 64, 8, 4, true>(a, s);
