@@ -554,6 +554,31 @@ __device__ __forceinline__ double gemm_tile_pipe(const GemmArgs& a, int64_t m0, 
 }
 
 
+// The probability check of a thread whose FP32 pair has left the finite range
+// (an infinite bin, whose TwoSum error is NaN, or a sum beyond FP32's largest
+// value): the same groups again, from the outputs the thread has written, in
+// FP64 as gemm_tile adds them.  Rare, out of line.
+template <int G, int R>
+__device__ __noinline__ double band_sum_again(const float* out, const uint64_t* roff, int first, int step, int bm) {
+  double sum = 0.0;
+  for (int r0 = first; r0 < bm; r0 += step)
+    for (int r = r0; r < r0 + R; r += G) {
+      float g0 = 0.f, g1 = 0.f;
+      for (int g = 0; g < G; ++g) {
+        const float4 v = *reinterpret_cast<const float4*>(out + roff[r + g]);
+        if constexpr (G == 2) {
+          g0 = (g0 + v.x) + v.y;
+          g1 = (g1 + v.z) + v.w;
+        } else {
+          g0 += (v.x + v.y) + (v.z + v.w);
+        }
+      }
+      sum += double(g0);
+      if constexpr (G == 2) sum += double(g1);
+    }
+  return sum;
+}
+
 // Bands: steps of a short shared index (K = 1, 4 or 16) with contiguous output
 // columns (vec4) and FP32 output write far more than they read or multiply.
 // In plain tiles a thread stores a few values after a chain of dependent
@@ -641,8 +666,9 @@ __device__ __forceinline__ double gemm_band_k(const GemmArgs& a, int64_t m0, int
     two_sum_add(s_hi, s_lo, g0);
     if constexpr (G == 2) two_sum_add(s_hi, s_lo, g1);
   }
+  const double sum = isfinite(s_hi) ? double(s_hi) + double(s_lo) : band_sum_again<G, G>(out, roff, rg * G, nrg * G, bm);
   __syncthreads();                                   // the next band may reuse the shared memory
-  return double(s_hi) + double(s_lo);
+  return sum;
 }
 // K = 16: both operands in shared memory, k-major; 8 rows x 4 columns per
 // thread and round, the multiply-adds of two rows in one instruction (four B
@@ -727,8 +753,9 @@ __device__ __forceinline__ double gemm_band_16(const GemmArgs& a, int64_t m0, in
       }
     }
   }
+  const double sum = isfinite(s_hi) ? double(s_hi) + double(s_lo) : band_sum_again<G, 8>(out, roff, rg * 8, nrg * 8, bm);
   __syncthreads();                                   // the next band may reuse the shared memory
-  return double(s_hi) + double(s_lo);
+  return sum;
 }
 
 template <int G, bool CG>
