@@ -503,8 +503,10 @@ sqc_status attribute_all(sqc_ctx* ctx, Circuit* c, const void* const* probs, sqc
       }
       d.L1 = L1;
       d.L2 = L2;
-      d.vec = L1 == 5 && L2 == 3 && dtype != SQC_F64 && (reinterpret_cast<uintptr_t>(src[i]) % 16) == 0;
-      d.async2 = d.vec && kout == 0 && kin >= 1 && S <= 32;
+      // (without incoming edges a 4-state-per-thread CTA takes four tiles)
+      d.vec = L1 == 5 && L2 == 3 && dtype != SQC_F64 && (reinterpret_cast<uintptr_t>(src[i]) % 16) == 0 &&
+              (kin > 0 || n + 2 * kout >= L1 + L2 + 2);
+      d.async2 = d.vec && kout == 0 && kin >= 1 && S <= 32 && n >= kRingL1 + kRingL2;
       // without outgoing edges A_i is as large as p_i and the bit-reversed
       // write runs (2^L2 states) set the speed: the double-buffered form
       // takes 16 x 32 tiles (64-byte reads, 128-byte writes) in a ring of
