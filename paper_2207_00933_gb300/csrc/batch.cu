@@ -77,6 +77,8 @@ __device__ __forceinline__ double run_tile(const BatchStep& st, int64_t tile, fl
   return gemm_tile<BM, BN, TM, TN, CH, BK, kOpThreads, true>(st.a, m0, n0, smem, smem + BK * (BM + 4), C);
 }
 
+constexpr int64_t kLead = 2;
+
 __global__ void __launch_bounds__(kOpThreads, 3) batch_kernel(BatchLaunch L) {
   pdl_wait();      // the previous kernel on the stream has completed
   pdl_trigger();   // the next one may start launching
@@ -87,17 +89,22 @@ __global__ void __launch_bounds__(kOpThreads, 3) batch_kernel(BatchLaunch L) {
   __shared__ bool is_last;
   __shared__ int skip;                        // -1: no more items
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // Items are claimed one ahead, so that an item's number and contents are on
-  // their way while the one before it is worked on.  Every CTA works through
-  // its claims in list order, so the earliest unfinished item is never held
-  // up by a later one and the schedule still cannot deadlock.
+  // While the list is long, items are claimed ahead, so that an item's number
+  // and contents are on their way while the one before it is worked on.  Its
+  // last kLead items per CTA (all of a short list) are claimed when the CTA is
+  // free: claimed ahead they would wait behind the item at hand while other
+  // CTAs are idle.  Every CTA works through its claims in list order, so the
+  // earliest unfinished item is never held up by a later one and the schedule
+  // still cannot deadlock.
   auto claim = [&]() -> int64_t {
     return int64_t(atomicAdd(reinterpret_cast<unsigned long long*>(L.head), 1ull));
   };
-  int64_t id = 0, next = 0;                   // thread 0: this item's number and the next one's
+  constexpr int64_t kNone = -1;
+  const int64_t ahead_to = L.n_items - kLead * int64_t(gridDim.x);   // items before it are claimed ahead
+  int64_t id = 0, next = kNone;               // thread 0: this item's number and the next one's
   if (threadIdx.x == 0) {
     id = claim();
-    next = claim();
+    if (id < ahead_to) next = claim();
     if (id < L.n_items) items[0] = L.items[id];
   }
   for (int p = 0;; p ^= 1) {
@@ -133,26 +140,29 @@ __global__ void __launch_bounds__(kOpThreads, 3) batch_kernel(BatchLaunch L) {
             have[k] = ld_acquire(L.counts + dep);
           }
         }
-        if (item.type == kItemMerge) md = L.mdescs[item.idx];
         skip = *static_cast<volatile int*>(L.abort) ? 1 : 0;    // one decision for the whole CTA
       }
     }
     __syncthreads();
     const int sk = skip;
     if (sk < 0) break;
-    if (threadIdx.x == 0) {
+    int64_t after = kNone;
+    if (threadIdx.x == 0 && next != kNone) {
       if (next < L.n_items) {
         const char* src = reinterpret_cast<const char*>(L.items + next);
         const uint32_t dst = uint32_t(__cvta_generic_to_shared(&items[p ^ 1]));
         asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
         asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst + 16), "l"(src + 16) : "memory");
       }
-      id = sk ? L.n_items : next;             // after an abort: drain
-      next = claim();
+      if (next < ahead_to) after = claim();
     }
     const BatchStep* sums = nullptr;          // a last step with a probability sum
     if (!sk) {
       if (item.type == kItemMerge) {
+        static_assert(sizeof(MergeDesc) % 8 == 0 && sizeof(MergeDesc) / 8 <= kOpThreads, "a thread per word");
+        if (threadIdx.x < sizeof(MergeDesc) / 8)
+          reinterpret_cast<uint64_t*>(&md)[threadIdx.x] = reinterpret_cast<const uint64_t*>(L.mdescs + item.idx)[threadIdx.x];
+        __syncthreads();
         for (int b = 0; b < item.count; ++b) {
           if (md.tiled) merge_tile(md, item.tile + b, smem);
           else merge_block(md, item.tile + b);
@@ -197,7 +207,18 @@ __global__ void __launch_bounds__(kOpThreads, 3) batch_kernel(BatchLaunch L) {
         atomicAdd(L.counts + item.out, 1u);
       }
     }
-    if (threadIdx.x == 0) asm volatile("cp.async.wait_all;" ::: "memory");
+    if (threadIdx.x == 0) {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      if (sk) {
+        id = L.n_items;                       // after an abort: drain
+      } else if (next != kNone) {
+        id = next;
+        next = after;
+      } else {
+        id = claim();
+        if (id < L.n_items) items[p ^ 1] = L.items[id];
+      }
+    }
   }
   // the last CTA out re-arms the schedule for the next launch
   if (threadIdx.x == 0) {
