@@ -79,7 +79,7 @@ __device__ __forceinline__ double run_tile(const BatchStep& st, int64_t tile, fl
 
 constexpr int64_t kLead = 2;
 
-__global__ void __launch_bounds__(kOpThreads, 3) batch_kernel(BatchLaunch L) {
+__global__ void __launch_bounds__(kOpThreads, kBatchCtasPerSm) batch_kernel(BatchLaunch L) {
   pdl_wait();      // the previous kernel on the stream has completed
   pdl_trigger();   // the next one may start launching
   extern __shared__ __align__(16) float smem[];

@@ -309,6 +309,7 @@ struct BatchLaunch {
   void* out;                 // output of the steps marked from_launch (a single-query launch)
   double* total;             // their probability sum (nullable)
 };
+constexpr int kBatchCtasPerSm = 3;         // resident CTAs of the work list's launch
 cudaError_t launch_batch(const BatchLaunch& L, int grid, cudaStream_t s);
 // The merges of a batch as a launch of their own ahead of the steps': n items
 // (type merge, no dependencies), one per CTA; tiled: some descriptor is.
