@@ -5,23 +5,24 @@
 //
 // The host flattens every query's contraction bands and tiles into one work
 // list ordered by dependency level.  Persistent CTAs claim items in list order
-// from a global head counter, one ahead of the item they work on.  Every
-// tensor has a completion counter; an item waits (bounded) until the counters
-// of its input tensors reach their expected item counts, does its work, then
-// bumps the counter of the tensor it wrote.  An item only ever waits for items
-// earlier in the list, and every CTA works through its claims in order, so the
-// earliest unfinished item always runs and the schedule cannot deadlock.  The
-// last CTA to leave re-arms the head and the counters, so the same launch can
-// be replayed (e.g. from a CUDA graph).  On a wait timeout the kernel raises
-// an abort flag that makes every CTA drain quickly and records an error code.
+// from a global head counter, ahead of the item they work on while many are
+// left.  Every tensor has a completion counter; an item waits (bounded) until
+// the counters of its input tensors reach their expected item counts, does its
+// work, then bumps the counter of the tensor it wrote.  An item only ever waits
+// for items earlier in the list, and every CTA works through its claims in
+// order, so the earliest unfinished item always runs and the schedule cannot
+// deadlock.  The last CTA to leave re-arms the head and the counters, so the
+// same launch can be replayed (e.g. from a CUDA graph).  On a wait timeout the
+// kernel raises an abort flag that makes every CTA drain quickly and records an
+// error code.
 //
 // Bound: the latency of its items (operands, map entries and counters from
 // L2), so three CTAs per SM although the 64 x 64 tiles then spill.  256 queries
 // of 10 to 20 active qubits over four circuits (165 MB of bins, 863 MB of
 // states merged from L2): 162 us, 66 of them the merges (180 with two CTAs per
 // SM, 158 with four, where longer shared indices lose: 64 queries of K = 64
-// steps 210, 197 and 200 us); one launch with a merge block or a 32 x 32 tile
-// per item took 833 us.
+// steps 210, 197 and 200 us, 190 since a list's last items are claimed late);
+// one launch with a merge block or a 32 x 32 tile per item took 833 us.
 #include "device_ops.cuh"
 
 namespace sqc {
@@ -77,6 +78,8 @@ __device__ __forceinline__ double run_tile(const BatchStep& st, int64_t tile, fl
   return gemm_tile<BM, BN, TM, TN, CH, BK, kOpThreads, true>(st.a, m0, n0, smem, smem + BK * (BM + 4), C);
 }
 
+// Items per CTA at the end of a list that are not claimed ahead (1, 2, 4: 256
+// queries 169, 163, 164 us; 64 with the pyramid 195, 190, 190).
 constexpr int64_t kLead = 2;
 
 __global__ void __launch_bounds__(kOpThreads, kBatchCtasPerSm) batch_kernel(BatchLaunch L) {
@@ -238,9 +241,13 @@ __global__ void __launch_bounds__(kOpThreads, kBatchCtasPerSm) batch_kernel(Batc
 }
 
 // The merges of a level, one work item (some blocks of one descriptor) per
-// CTA.  On their own because they need a quarter of the steps' registers:
-// eight CTAs per SM cover the descriptor and item loads and the short chains
-// of each sum, where the steps' kernel holds two.  The states come from L2
+// CTA.  On their own because they need 32 registers where the steps' kernel
+// needs 80: eight CTAs per SM cover the descriptor and item loads and the short
+// chains of each sum, where that one holds three.  The price: a level whose
+// merges take longer than its steps has no steps to hide them (16 queries with
+// runs of 2^12 states and more over 16 MB: 54 + 30 us, 64 us together in one
+// list).  With the long merges in the list, 256 queries took 163-197 us for
+// 162.  The states come from L2
 // (the resident tensors of a level's circuits fit it), so L2 bandwidth is the
 // bound.
 template <bool TILED>

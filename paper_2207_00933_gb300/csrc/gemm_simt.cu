@@ -54,18 +54,19 @@ __global__ void __launch_bounds__(kPipeThreads, 3) gemm_pipe_kernel(GemmArgs a) 
 // Steps of at most 1024 outputs and 16 shared terms, one after the other in
 // one CTA: what a long chain of narrow subcircuits contracts to (a 59-block
 // chain has 55 such steps in a row).  A launch each costs the host and the
-// GPU about 3 us; here a step is one round of loads from L2 (both operand
-// rows and the two map entries of an output together), its multiply-adds and
-// a store.  k runs upwards with gemm_tile's zero term below 16: the values are
-// the same bit for bit.  Bound: the latency of L2.
+// GPU about 3 us; here an output is one round of loads from L2 (both operand
+// rows and the two map entries together), its multiply-adds and a store, and a
+// thread's outputs follow each other: one round per 256 outputs of a step.  k
+// runs upwards with gemm_tile's zero term below 16: the values are the same bit
+// for bit.  Bound: the latency of L2.
 __global__ void __launch_bounds__(kThreads) gemm_small_run_kernel(const __grid_constant__ SmallRun r) {
   pdl_wait();      // the previous kernel on the stream has completed
   pdl_trigger();   // the next one may start launching
   for (int i = 0; i < r.n; ++i) {
     const SmallStep& st = r.s[i];
     const int nl = st.n_log2, outs = 1 << (st.m_log2 + nl), K = 1 << st.k_log2;
-    // every thread's offsets and operands before any store: an output's place
-    // may not depend on the step before, but its operands do
+    // (a step's output is none of its operands; the barrier below orders it
+    // before the next step's loads)
     for (int o = threadIdx.x; o < outs; o += kThreads) {
       const int row = o >> nl, col = o & ((1 << nl) - 1);
       const uint64_t at = __ldg(st.rowmap + row) + __ldg(st.colmap + col);

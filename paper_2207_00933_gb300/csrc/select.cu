@@ -1511,8 +1511,9 @@ struct NoSource {
 };
 
 // The sampled chunk of stratum s: a fixed pseudo-random multiple of 4 inside
-// it (a mixing function of the index, so that no period of the input lines
-// up with the sample).
+// it, so that no period of the input lines up with the sample (s times the
+// first 32-bit prime of xxHash, then the first two steps of its final mix,
+// by Y. Collet).
 __device__ __forceinline__ uint64_t sample_at(unsigned s, uint64_t span) {
   unsigned h = s * 0x9E3779B1u;
   h ^= h >> 15;
@@ -2016,9 +2017,10 @@ select_resident_kernel(const void* x, int aligned, uint64_t n, uint64_t per, uns
     // (cp.async, kLoadRing - 1 rounds ahead, no barrier): one CTA per SM is
     // bound by the loads in flight, and plain loads by the small L1 that is
     // left beside this much shared memory (2^22 FP64 values from L2, the whole
-    // selection: 35-42 us with plain loads, 25-32 us so; FP32 the same).  The
-    // loop bound is the same for the whole CTA: warp_hist_add needs every lane
-    // of the warp.
+    // selection: 35-42 us with plain loads, 25-32 us so).  FP64 only: FP32,
+    // half the bytes, gains nothing (4553 values a CTA 15.1 -> 15.4 us) and
+    // keeps plain loads.  The loop bound is the same for the whole CTA:
+    // warp_hist_add needs every lane of the warp.
     using Word = std::conditional_t<F64, unsigned long long, unsigned>;
     unsigned char* ring = reinterpret_cast<unsigned char*>(keys + per);
     const bool ringed = F64 && aligned && T.ring;
