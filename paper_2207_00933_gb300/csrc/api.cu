@@ -1247,8 +1247,8 @@ sqc_status finalize_plan(sqc_ctx* ctx, Plan* P) {
   // Few outputs over long runs, a warp per output: a query's whole merge when
   // every subcircuit's is (merge_is_long), else a launch of its own for those of
   // 2^14 states and more, whose warps would outlast the others by more than the
-  // launch costs (8 outputs of 2^19 states beside others: the merge 570-850 us,
-  // 157 so).
+  // launch costs (8 outputs of 2^19 states beside others: the merge 487 us, 149
+  // so).
   int64_t blocks = 0, long_outputs = 0;
   bool any_tiled = false, all_long = true;
   for (const MergeDesc& d : P->merge_host) all_long = all_long && merge_is_long(d);

@@ -462,9 +462,10 @@ __device__ __forceinline__ void fma2(float2& d, float2 a, float2 b) {
 // two CTAs per SM, 1.4% faster at 4096 x 4096 x 256 and 11% slower at
 // 4096 x 2048 x 256; A doubled in shared memory to save the register moves,
 // 13% slower.)
-// 4096 x 4096 x 256: 178 us, 48 TFLOP/s of the 75 that packed multiply-adds
+// 4096 x 4096 x 256: 164 us, 52 TFLOP/s of the 75 that packed multiply-adds
 // reach from registers (gemm_tile's unbuffered stages and scalar loads: 218
-// us); 4096 x 2048 x 256 131 -> 95 us, 4096 x 2048 x 64 47 -> 37 us.
+// us).  Before the epilogue read its map entries first it took 178 us, 4096 x
+// 2048 x 256 131 -> 95 us and 4096 x 2048 x 64 47 -> 37 us.
 constexpr int kPipeK = 16;
 template <int BM, int BN>
 constexpr int gemm_pipe_smem_floats() {
