@@ -333,31 +333,38 @@ __device__ __forceinline__ double gemm_tile(const GemmArgs& a, int64_t m0, int64
     if constexpr (CG) return __ldcg(reinterpret_cast<const float4*>(p));
     else return __ldg(reinterpret_cast<const float4*>(p));
   };
+  // Row and first shared index of word i: a warp takes 8 rows x 4 words, whose
+  // transposed stores meet in two lanes per bank (2 rows x 16 words, for a
+  // stage of 64, in eight: 128 x 128 outputs of K = 256 with their merge 17.1
+  // us, 14.8 so; 64 queries of K = 64 steps 189 -> 179).
+  static_assert(BM % 8 == 0 && BN % 8 == 0 && kQ % 4 == 0, "whole warps of words");
+  auto row_of = [](int i) -> int { return ((i >> 2) & 7) + 8 * ((i >> 5) / (kQ / 4)); };
+  auto k_of = [](int i) -> int { return 4 * ((i & 3) + 4 * ((i >> 5) % (kQ / 4))); };
   for (int64_t k0 = 0; k0 < a.K; k0 += kBK) {
     if (a.K >= 4) {
       float4 ra[kLA], rb[kLB];
 #pragma unroll
       for (int u = 0; u < kLA; ++u) {
-        const int i = tid + u * kThreads, r = i / kQ, kk = 4 * (i % kQ);
+        const int i = tid + u * kThreads, r = row_of(i), kk = k_of(i);
         ra[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (i < BM * kQ && m0 + r < a.M && k0 + kk < a.K) ra[u] = ld4(a.A + (m0 + r) * a.K + k0 + kk);
       }
 #pragma unroll
       for (int u = 0; u < kLB; ++u) {
-        const int i = tid + u * kThreads, r = i / kQ, kk = 4 * (i % kQ);
+        const int i = tid + u * kThreads, r = row_of(i), kk = k_of(i);
         rb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (i < BN * kQ && n0 + r < a.N && k0 + kk < a.K) rb[u] = ld4(a.B + (n0 + r) * a.K + k0 + kk);
       }
 #pragma unroll
       for (int u = 0; u < kLA; ++u) {
-        const int i = tid + u * kThreads, r = i / kQ, kk = 4 * (i % kQ);
+        const int i = tid + u * kThreads, r = row_of(i), kk = k_of(i);
         if (i < BM * kQ) {
           As[kk][r] = ra[u].x; As[kk + 1][r] = ra[u].y; As[kk + 2][r] = ra[u].z; As[kk + 3][r] = ra[u].w;
         }
       }
 #pragma unroll
       for (int u = 0; u < kLB; ++u) {
-        const int i = tid + u * kThreads, r = i / kQ, kk = 4 * (i % kQ);
+        const int i = tid + u * kThreads, r = row_of(i), kk = k_of(i);
         if (i < BN * kQ) {
           Bs[kk][r] = rb[u].x; Bs[kk + 1][r] = rb[u].y; Bs[kk + 2][r] = rb[u].z; Bs[kk + 3][r] = rb[u].w;
         }
