@@ -495,7 +495,9 @@ sqc_status attribute_all(sqc_ctx* ctx, Circuit* c, const void* const* probs, sqc
       for (;;) {
         const int64_t slots = S << (L1 + L2 + 1), tiles_next = ((int64_t(1) << (n - L1 - L2)) << (2 * kout)) >> 1;
         if (L1 + L2 >= n || (slots << kout) > tile_reads ||
-            slots > (tiles_next >= kAttrManyTiles ? kAttrSmemMax / 4 : kAttrSlots))
+            slots > (tiles_next >= 2 * kAttrManyTiles ? kAttrSmemMax / 4
+                     : tiles_next >= kAttrManyTiles   ? kAttrSmemMax / 8
+                                                      : kAttrSlots))
           break;
         if (L2 < 3) ++L2;
         else if (L1 < 5) ++L1;
