@@ -21,7 +21,8 @@
 // of 10 to 20 active qubits over four circuits (165 MB of bins, 863 MB of
 // states merged from L2): 162 us, 66 of them the merges (180 with two CTAs per
 // SM, 158 with four, where longer shared indices lose: 64 queries of K = 64
-// steps 210, 197 and 200 us, 190 since a list's last items are claimed late);
+// steps 210, 197 and 200 us, 179 since a list's last items are claimed late and
+// a 64-deep stage's stores spread over the banks);
 // one launch with a merge block or a 32 x 32 tile per item took 833 us.
 #include "device_ops.cuh"
 
